@@ -109,15 +109,15 @@ __device__ __forceinline__ void lbs_warp(const FieldParams &P, const float *__re
 // ------------------------------------------------------- positional encoding
 // Sec. 4.3: gamma(x) = [x^, w_k sin(2^k pi x^), w_k cos(2^k pi x^)]_{k<L} with
 // x^ the point normalised to [-1, 1] over the box and w_k the truncated Hann
-// weight of band k.  Writes kResGammaPad values (zero padded).
-__device__ __forceinline__ void pos_enc(const FieldParams &P, float x0, float x1, float x2, float *__restrict__ g,
-                                        int stride) {
+// weight of band k.  put(k, v) receives kResGammaPad values (zero padded).
+template <typename Put>
+__device__ __forceinline__ void pos_enc(const FieldParams &P, float x0, float x1, float x2, Put &&put) {
   const float h0 = (x0 - P.box_c[0]) * P.box_ih[0];
   const float h1 = (x1 - P.box_c[1]) * P.box_ih[1];
   const float h2 = (x2 - P.box_c[2]) * P.box_ih[2];
-  g[0] = h0;
-  g[stride] = h1;
-  g[2 * stride] = h2;
+  put(0, h0);
+  put(1, h1);
+  put(2, h2);
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const float sc = (float)(1 << k);
@@ -126,16 +126,21 @@ __device__ __forceinline__ void pos_enc(const FieldParams &P, float x0, float x1
     sincospif(sc * h1, &sb, &cb);
     sincospif(sc * h2, &sd, &cd);
     const float w = (k < P.res_freqs) ? P.hann[k] : 0.f;
-    float *q = g + (3 + 6 * k) * stride;
-    q[0] = w * sa;
-    q[stride] = w * sb;
-    q[2 * stride] = w * sd;
-    q[3 * stride] = w * ca;
-    q[4 * stride] = w * cb;
-    q[5 * stride] = w * cd;
+    const int q = 3 + 6 * k;
+    put(q, w * sa);
+    put(q + 1, w * sb);
+    put(q + 2, w * sd);
+    put(q + 3, w * ca);
+    put(q + 4, w * cb);
+    put(q + 5, w * cd);
   }
 #pragma unroll
-  for (int j = 39; j < kResGammaPad; ++j) g[j * stride] = 0.f;
+  for (int j = 39; j < kResGammaPad; ++j) put(j, 0.f);
+}
+
+__device__ __forceinline__ void pos_enc(const FieldParams &P, float x0, float x1, float x2, float *__restrict__ g,
+                                        int stride) {
+  pos_enc(P, x0, x1, x2, [=](int k, float v) { g[k * stride] = v; });
 }
 
 // ------------------------------------------------------------- hash encoding
@@ -235,9 +240,9 @@ __device__ __forceinline__ void hash_level(const FieldParams &P, int l, float p0
   }
 }
 
-// enc (a column with the given stride): 2 features per level, zero beyond 2L.  Returns whether x is inside the box.
-__device__ __forceinline__ bool hash_encode(const FieldParams &P, float x0, float x1, float x2, float *__restrict__ enc,
-                                            int stride) {
+// put(k, v): 2 features per level, zero beyond 2L.  Returns whether x is inside the box.
+template <typename Put>
+__device__ __forceinline__ bool hash_encode(const FieldParams &P, float x0, float x1, float x2, Put &&put) {
   float p0 = (x0 - P.bmin[0]) * P.inv_box[0];
   float p1 = (x1 - P.bmin[1]) * P.inv_box[1];
   float p2 = (x2 - P.bmin[2]) * P.inv_box[2];
@@ -250,52 +255,100 @@ __device__ __forceinline__ bool hash_encode(const FieldParams &P, float x0, floa
   for (int l = 0; l < P.L; ++l) {
     float a, b;
     hash_level(P, l, p0, p1, p2, a, b);
-    enc[(2 * l) * stride] = inside ? a : 0.f;
-    enc[(2 * l + 1) * stride] = inside ? b : 0.f;
+    put(2 * l, inside ? a : 0.f);
+    put(2 * l + 1, inside ? b : 0.f);
   }
   for (int l = P.L; l < kMaxLevels; ++l) {
-    enc[(2 * l) * stride] = 0.f;
-    enc[(2 * l + 1) * stride] = 0.f;
+    put(2 * l, 0.f);
+    put(2 * l + 1, 0.f);
   }
   return inside;
 }
 
+__device__ __forceinline__ bool hash_encode(const FieldParams &P, float x0, float x1, float x2, float *__restrict__ enc,
+                                            int stride) {
+  return hash_encode(P, x0, x1, x2, [=](int k, float v) { enc[k * stride] = v; });
+}
+
 // -------------------------------------------------------- float32 MLP layers
-// y = W x + b with W stored transposed ([in][out], out a multiple of 4) in
-// shared memory and read as broadcast float4 (all threads of the block read
-// the same weight).  Each thread keeps its activations in its own column of a
-// shared-memory buffer, col[k * stride] (stride = threads per block), so the
-// loop over inputs is a runtime loop; the 64 accumulators live in registers.
-template <int OUT>
-__device__ __forceinline__ void dense_acc_f32(const float *__restrict__ Wt, const float *__restrict__ col, int in,
-                                              int stride, float (&y)[OUT]) {
-#pragma unroll 2
+// A warp takes a tile of 32 samples.  Activations of the tile lie in shared memory as rows of
+// 32 samples (one row an input), the row's eight 16-byte chunks permuted by the row number so
+// that every access below is free of bank conflicts; weights are the transposed blob ([in][out])
+// in shared memory.
+constexpr int kTileGamma = 40;   // rows of gamma(x_skel) in a tile: the 39 used and a zero row
+__device__ __forceinline__ int tile_at(int row, int smp) {
+  return row * 32 + ((((smp >> 2) ^ (row >> 2)) & 7) << 2) + (smp & 3);
+}
+
+// acc[i][j] += sum_k x[k][sample 8 (lane & 3) + i] W[k][out], out = 4 (lane >> 2) + j for j < 4
+// and 28 more for the others, k in increasing order.  Each lane holds an 8 x 8 block of the
+// 32 x 64 outputs, so one k costs two 16-byte loads of x, two of W and 64 FMAs: with one thread a
+// sample (one broadcast load of W per four FMAs) the shared-memory pipe held the FMA pipe to a
+// quarter of its rate.
+__device__ __forceinline__ void tile_acc(const float *__restrict__ Wt, const float *__restrict__ x, int in,
+                                         float (&acc)[8][8]) {
+  const int lane = threadIdx.x & 31, a = lane & 3, b = lane >> 2;
+  const float4 *w = reinterpret_cast<const float4 *>(Wt) + b;
+#pragma unroll 4
   for (int k = 0; k < in; ++k) {
-    const float xk = col[k * stride];
-    const float4 *row = reinterpret_cast<const float4 *>(Wt + k * OUT);
+    const float4 *row = reinterpret_cast<const float4 *>(x + k * 32);
+    const int f = (k >> 2) & 7;
+    const float4 xa = row[(2 * a) ^ f], xb = row[(2 * a + 1) ^ f];
+    const float4 wa = w[k * 16], wb = w[k * 16 + 8];
+    const float xs[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+    const float ws[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
-    for (int j = 0; j < OUT / 4; ++j) {
-      const float4 w = row[j];
-      y[4 * j + 0] = fmaf(xk, w.x, y[4 * j + 0]);
-      y[4 * j + 1] = fmaf(xk, w.y, y[4 * j + 1]);
-      y[4 * j + 2] = fmaf(xk, w.z, y[4 * j + 2]);
-      y[4 * j + 3] = fmaf(xk, w.w, y[4 * j + 3]);
-    }
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(xs[i], ws[j], acc[i][j]);
   }
 }
 
-template <int OUT>
-__device__ __forceinline__ void dense_f32(const float *__restrict__ Wt, const float *__restrict__ b,
-                                          const float *__restrict__ col, int in, int stride, float (&y)[OUT]) {
+// h = relu(W [x | x2] + bias) for the warp's tile; h may be x (every lane has read x by then).
+__device__ __forceinline__ void tile_layer(const float *__restrict__ Wt, const float *__restrict__ bias, const float *x,
+                                           int in, const float *x2, int in2, float *h) {
+  const int lane = threadIdx.x & 31, a = lane & 3, b = lane >> 2;
+  float acc[8][8];
 #pragma unroll
-  for (int j = 0; j < OUT; ++j) y[j] = b[j];
-  dense_acc_f32<OUT>(Wt, col, in, stride, y);
+  for (int j = 0; j < 8; ++j) {
+    const float v = bias[4 * b + j + (j >= 4 ? 28 : 0)];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i][j] = v;
+  }
+  tile_acc(Wt, x, in, acc);
+  if (in2) tile_acc(Wt + in * kWidth, x2, in2, acc);
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const int o = 4 * b + j + (j >= 4 ? 28 : 0);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float4 v;
+      v.x = fmaxf(acc[4 * q][j], 0.f);
+      v.y = fmaxf(acc[4 * q + 1][j], 0.f);
+      v.z = fmaxf(acc[4 * q + 2][j], 0.f);
+      v.w = fmaxf(acc[4 * q + 3][j], 0.f);
+      *reinterpret_cast<float4 *>(h + tile_at(o, 8 * a + 4 * q)) = v;
+    }
+  }
+  __syncwarp();
 }
 
-template <int N>
-__device__ __forceinline__ void store_relu(const float (&y)[N], float *__restrict__ col, int stride) {
+// The four outputs of this lane's sample from 64 inputs.
+__device__ __forceinline__ void tile_out4(const float *__restrict__ Wt, const float *__restrict__ b, const float *x,
+                                          float (&y)[4]) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int j = 0; j < N; ++j) col[j * stride] = fmaxf(y[j], 0.f);
+  for (int j = 0; j < 4; ++j) y[j] = b[j];
+#pragma unroll 8
+  for (int k = 0; k < kWidth; ++k) {
+    const float xk = x[tile_at(k, lane)];
+    const float4 w = reinterpret_cast<const float4 *>(Wt)[k];
+    y[0] = fmaf(xk, w.x, y[0]);
+    y[1] = fmaf(xk, w.y, y[1]);
+    y[2] = fmaf(xk, w.z, y[2]);
+    y[3] = fmaf(xk, w.w, y[3]);
+  }
 }
 
 // The output activations with the accurate expf / log1pf and an IEEE division: rgb =
@@ -305,42 +358,32 @@ __device__ __forceinline__ void store_relu(const float (&y)[N], float *__restric
 __device__ __forceinline__ float sigmoidf_(float o) { return 1.f / (1.f + expf(-o)); }
 __device__ __forceinline__ float softplusf_(float o) { return fmaxf(o, 0.f) + log1pf(expf(-fabsf(o))); }
 
-// Residual MLP (Sec. 4.3, Fig. S3) in float32.  gcol holds gamma(x_skel)
-// (kResGammaPad rows), hcol is the 64-row scratch column; returns x_res.
-// bias1 holds b1 + W_Omega Omega (the pose folded into the first layer).
+// Residual MLP (Sec. 4.3, Fig. S3) in float32 of the warp's tile.  g holds gamma(x_skel)
+// (kTileGamma rows), h is a 64-row buffer; o[0..2] is x_res of this lane's sample.
+// bias1 holds b1 + W_Omega Omega (the pose folded into the first layer).  Warp-collective.
 __device__ __forceinline__ void residual_f32(const FieldParams &P, const float *__restrict__ W,
-                                             const float *__restrict__ bias1, const float *__restrict__ gcol,
-                                             float *__restrict__ hcol, int stride, float &r0, float &r1, float &r2) {
-  float y[kWidth];
-  dense_f32<kWidth>(W + P.lay.r1, bias1, gcol, kResGammaPad, stride, y);
-  store_relu(y, hcol, stride);
-  dense_f32<kWidth>(W + P.lay.r2, W + P.lay.r2b, hcol, kWidth, stride, y);
-  store_relu(y, hcol, stride);
-  dense_f32<kWidth>(W + P.lay.r3, W + P.lay.r3b, hcol, kWidth, stride, y);
-  store_relu(y, hcol, stride);
+                                             const float *__restrict__ bias1, const float *g, float *h,
+                                             float (&o)[4]) {
+  __syncwarp();   // the lanes' gamma columns
+  tile_layer(W + P.lay.r1, bias1, g, kTileGamma, nullptr, 0, h);
+  tile_layer(W + P.lay.r2, W + P.lay.r2b, h, kWidth, nullptr, 0, h);
+  tile_layer(W + P.lay.r3, W + P.lay.r3b, h, kWidth, nullptr, 0, h);
   // layer 4 sees [h3, gamma]: the transposed rows of h3, then those of gamma
-  dense_f32<kWidth>(W + P.lay.r4, W + P.lay.r4b, hcol, kWidth, stride, y);
-  dense_acc_f32<kWidth>(W + P.lay.r4 + kWidth * kWidth, gcol, kResGammaPad, stride, y);
-  store_relu(y, hcol, stride);
-  float o[4];
-  dense_f32<4>(W + P.lay.r5, W + P.lay.r5b, hcol, kWidth, stride, o);
-  r0 = o[0];
-  r1 = o[1];
-  r2 = o[2];
+  tile_layer(W + P.lay.r4, W + P.lay.r4b, h, kWidth, g, kTileGamma, h);
+  tile_out4(W + P.lay.r5, W + P.lay.r5b, h, o);
+  __syncwarp();   // h is free again
 }
 
-// Canonical MLP (MLP_nerf, Sec. 4.4) in float32 on the encoding held in hcol
-// rows 0..31; returns the 4 raw outputs.
-__device__ __forceinline__ void canonical_f32(const FieldParams &P, const float *__restrict__ W,
-                                              float *__restrict__ hcol, int stride, float (&o)[4]) {
-  float y[kWidth];
-  dense_f32<kWidth>(W + P.lay.c0, W + P.lay.c0b, hcol, kMlpIn, stride, y);
-  store_relu(y, hcol, stride);
-  for (int l = 0; l < P.hidden - 1; ++l) {
-    dense_f32<kWidth>(W + P.lay.ch[l], W + P.lay.chb[l], hcol, kWidth, stride, y);
-    store_relu(y, hcol, stride);
-  }
-  dense_f32<4>(W + P.lay.cl, W + P.lay.clb, hcol, kWidth, stride, o);
+// Canonical MLP (MLP_nerf, Sec. 4.4) in float32 on the encoding held in h's rows 0..31; o holds
+// the 4 raw outputs of this lane's sample.  Warp-collective.
+__device__ __forceinline__ void canonical_f32(const FieldParams &P, const float *__restrict__ W, float *h,
+                                              float (&o)[4]) {
+  __syncwarp();   // the lanes' encodings
+  tile_layer(W + P.lay.c0, W + P.lay.c0b, h, kMlpIn, nullptr, 0, h);
+  for (int l = 0; l < P.hidden - 1; ++l)
+    tile_layer(W + P.lay.ch[l], W + P.lay.chb[l], h, kWidth, nullptr, 0, h);
+  tile_out4(W + P.lay.cl, W + P.lay.clb, h, o);
+  __syncwarp();
 }
 
 }  // namespace nr

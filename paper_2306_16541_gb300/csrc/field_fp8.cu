@@ -20,6 +20,44 @@
 
 namespace nr {
 
+// ------------------------------------- float32 layers of the calibration, one point a thread
+// y = W x + b with W stored transposed ([in][out], out a multiple of 4) in
+// shared memory and read as broadcast float4 (all threads of the block read
+// the same weight).  Each thread keeps its activations in its own column of a
+// shared-memory buffer, col[k * stride] (stride = threads per block), so the
+// loop over inputs is a runtime loop; the 64 accumulators live in registers.
+template <int OUT>
+__device__ __forceinline__ void dense_acc_f32(const float *__restrict__ Wt, const float *__restrict__ col, int in,
+                                              int stride, float (&y)[OUT]) {
+#pragma unroll 2
+  for (int k = 0; k < in; ++k) {
+    const float xk = col[k * stride];
+    const float4 *row = reinterpret_cast<const float4 *>(Wt + k * OUT);
+#pragma unroll
+    for (int j = 0; j < OUT / 4; ++j) {
+      const float4 w = row[j];
+      y[4 * j + 0] = fmaf(xk, w.x, y[4 * j + 0]);
+      y[4 * j + 1] = fmaf(xk, w.y, y[4 * j + 1]);
+      y[4 * j + 2] = fmaf(xk, w.z, y[4 * j + 2]);
+      y[4 * j + 3] = fmaf(xk, w.w, y[4 * j + 3]);
+    }
+  }
+}
+
+template <int OUT>
+__device__ __forceinline__ void dense_f32(const float *__restrict__ Wt, const float *__restrict__ b,
+                                          const float *__restrict__ col, int in, int stride, float (&y)[OUT]) {
+#pragma unroll
+  for (int j = 0; j < OUT; ++j) y[j] = b[j];
+  dense_acc_f32<OUT>(Wt, col, in, stride, y);
+}
+
+template <int N>
+__device__ __forceinline__ void store_relu(const float (&y)[N], float *__restrict__ col, int stride) {
+#pragma unroll
+  for (int j = 0; j < N; ++j) col[j * stride] = fmaxf(y[j], 0.f);
+}
+
 constexpr int kF8Threads = 512;
 constexpr int kF8Warps = kF8Threads / 32;
 constexpr int kF8Row = 80;     // bytes per row of a K = 64 operand (64 + 16 pad)

@@ -79,10 +79,10 @@ __global__ void __launch_bounds__(256) march_kernel(CamParams cam, MarchParams m
 }
 
 // ------------------------------------------------------------- field (FP32)
-// One thread per sample; both MLPs' weights in shared memory (float32,
-// transposed), read as broadcast float4.  Writes (r, g, b, alpha) per sample
-// with alpha = (1 - exp(-sigma delta)) * min(S, 1) (Sec. 4.4 likelihood
-// augmentation), zero when the canonical point leaves the box.
+// A warp per tile of 32 samples: the gathers one sample per lane, both MLPs as the warp's
+// register-blocked layers (tile_layer) over the weights in shared memory (float32, transposed).
+// Writes (r, g, b, alpha) per sample with alpha = (1 - exp(-sigma delta)) * min(S, 1) (Sec. 4.4
+// likelihood augmentation), zero when the canonical point leaves the box.
 //
 // Two more modes build occupancy bitfields from the field itself (empty-space
 // skipping for subjects without ellipsoids, Sec. 2.3), one thread per cell of
@@ -93,100 +93,105 @@ __global__ void __launch_bounds__(256) march_kernel(CamParams cam, MarchParams m
 //                 (x_final: Eq. lbs then MLP_res, as for a sample).  The clamp
 //                 keeps a cell whose centre maps just outside the box while
 //                 other points of the cell map inside.
-// Cells are word-aligned per warp (occ_grid^3 is a multiple of 32 and so are
-// the block and the grid stride), so a warp ballot writes whole words.
-constexpr int kF32Threads = 192;
-constexpr int kF32ColRows = kWidth + kResGammaPad;   // per-thread activation column: h (64) then gamma (48)
+// occ_grid^3 is a multiple of 32, so a warp's tile is one word of the bitfield, written by its
+// ballot.
+//
+// Bound by the FMA pipe (28 K FMAs per sample of the tiny workload) at eight warps an SM: the
+// weights (100-135 KB) and 13.3 KB of activations a warp fill the shared memory.
+constexpr int kF32MaxThreads = 256;
+constexpr int kF32WarpFloats = (kWidth + kTileGamma) * 32;
 
 template <int MODE>
-__global__ void __launch_bounds__(kF32Threads, 1) field_f32_kernel(FieldParams P, const float4 *__restrict__ in,
-                                                                   uint32_t n_fixed, const uint32_t *__restrict__ n_dev,
-                                                                   float *__restrict__ out) {
+__global__ void __launch_bounds__(kF32MaxThreads, 1) field_f32_kernel(FieldParams P, const float4 *__restrict__ in,
+                                                                      uint32_t n_fixed,
+                                                                      const uint32_t *__restrict__ n_dev,
+                                                                      float *__restrict__ out) {
   extern __shared__ float4 smem4[];
   float *sW = reinterpret_cast<float *>(smem4);
   float *sG = sW + P.lay.total;
   float *sB1 = sG + kPoseSmem;
-  float *sCol = sB1 + kWidth;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  float *h = sB1 + kWidth + warp * kF32WarpFloats;   // this warp's activations: 64 rows, then gamma
+  float *g = h + kWidth * 32;
+  constexpr bool kCells = MODE == kModeDensity || MODE == kModePose;
+  const uint32_t n = kCells ? (uint32_t)P.occ_grid * P.occ_grid * P.occ_grid : (n_dev ? *n_dev : n_fixed);
+  const uint32_t n_tiles = (n + 31) / 32, slots = gridDim.x * warps;
+  // a launch with less than a tile per warp spreads its tiles over the SMs first
+  const uint32_t first = n_tiles < slots ? warp * gridDim.x + blockIdx.x : blockIdx.x * warps + warp;
+  if (n_tiles < slots && blockIdx.x >= n_tiles) return;   // no tile for any warp of the block
   for (int i = threadIdx.x; i < P.lay.total / 4; i += blockDim.x)
     reinterpret_cast<float4 *>(sW)[i] = __ldg(reinterpret_cast<const float4 *>(P.blob) + i);
   const float *sBox = stage_pose(P, sG, threadIdx.x, blockDim.x);
   for (int i = threadIdx.x; i < kWidth; i += blockDim.x) sB1[i] = P.bias1[i];
   __syncthreads();
-  const int stride = blockDim.x;
-  float *hcol = sCol + threadIdx.x;
-  float *gcol = hcol + kWidth * stride;
-  constexpr bool kCells = MODE == kModeDensity || MODE == kModePose;
-  float h[3] = {0.f, 0.f, 0.f};
+  auto put_h = [=](int k, float v) { h[tile_at(k, lane)] = v; };
+  auto put_g = [=](int k, float v) {
+    if (k < kTileGamma) g[tile_at(k, lane)] = v;
+  };
+  float hc[3] = {0.f, 0.f, 0.f};
   if (kCells) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) h[k] = __fdiv_rn(__fsub_rn(P.bmax[k], P.bmin[k]), (float)P.occ_grid);
+    for (int k = 0; k < 3; ++k) hc[k] = __fdiv_rn(__fsub_rn(P.bmax[k], P.bmin[k]), (float)P.occ_grid);
   }
-  const uint32_t n = kCells ? (uint32_t)P.occ_grid * P.occ_grid * P.occ_grid : (n_dev ? *n_dev : n_fixed);
-  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    float x0, x1, x2, delta = 0.f;
-    if (MODE == kModeRender) {
+  for (uint32_t tile = first; tile < n_tiles; tile += slots) {
+    const uint32_t j = tile * 32 + lane;
+    const bool valid = j < n;
+    float x0 = 0.f, x1 = 0.f, x2 = 0.f, delta = 0.f;
+    if (kCells) {
+      const uint32_t gr = (uint32_t)P.occ_grid;
+      x0 = __fadd_rn(P.bmin[0], __fmul_rn(__fadd_rn((float)(j % gr), 0.5f), hc[0]));
+      x1 = __fadd_rn(P.bmin[1], __fmul_rn(__fadd_rn((float)((j / gr) % gr), 0.5f), hc[1]));
+      x2 = __fadd_rn(P.bmin[2], __fmul_rn(__fadd_rn((float)(j / (gr * gr)), 0.5f), hc[2]));
+    } else if (valid && MODE == kModeRender) {
       const float4 s = in[j];
       x0 = s.x;
       x1 = s.y;
       x2 = s.z;
       delta = s.w;
-    } else if (MODE == kModeQuery) {
+    } else if (valid) {
       const float *q = reinterpret_cast<const float *>(in) + 3 * (size_t)j;
       x0 = q[0];
       x1 = q[1];
       x2 = q[2];
-    } else {
-      const uint32_t g = (uint32_t)P.occ_grid;
-      x0 = __fadd_rn(P.bmin[0], __fmul_rn(__fadd_rn((float)(j % g), 0.5f), h[0]));
-      x1 = __fadd_rn(P.bmin[1], __fmul_rn(__fadd_rn((float)((j / g) % g), 0.5f), h[1]));
-      x2 = __fadd_rn(P.bmin[2], __fmul_rn(__fadd_rn((float)(j / (g * g)), 0.5f), h[2]));
     }
+    float o[4];
     if (MODE == kModeDensity) {
-      hash_encode(P, x0, x1, x2, hcol, stride);
-      float o[4];
-      canonical_f32(P, sW, hcol, stride, o);
+      hash_encode(P, x0, x1, x2, put_h);
+      canonical_f32(P, sW, h, o);
       const unsigned word = __ballot_sync(0xffffffffu, softplusf_(o[3]) > P.occ_tau);
-      if ((threadIdx.x & 31) == 0) reinterpret_cast<uint32_t *>(out)[j >> 5] = word;
+      if (lane == 0) reinterpret_cast<uint32_t *>(out)[tile] = word;
       continue;
     }
     float s0, s1, s2, S;
     lbs_warp(P, sG, x0, x1, x2, s0, s1, s2, S, sBox);
     float f0 = s0, f1 = s1, f2 = s2;
-    if (MODE == kModePose) {
-      bool occ = false;
-      if (S >= P.occ_smin) {
-        if (P.res_enabled) {
-          pos_enc(P, s0, s1, s2, gcol, stride);
-          float r0, r1, r2;
-          residual_f32(P, sW, sB1, gcol, hcol, stride, r0, r1, r2);
-          f0 += r0;
-          f1 += r1;
-          f2 += r2;
-        }
-        // clamped to the grid as floats before the conversion (fmaxf maps NaN to 0)
-        const float top = (float)(P.occ_grid - 1);
-        const float c0 = fminf(fmaxf(floorf(__fdiv_rn(__fsub_rn(f0, P.bmin[0]), h[0])), 0.f), top);
-        const float c1 = fminf(fmaxf(floorf(__fdiv_rn(__fsub_rn(f1, P.bmin[1]), h[1])), 0.f), top);
-        const float c2 = fminf(fmaxf(floorf(__fdiv_rn(__fsub_rn(f2, P.bmin[2]), h[2])), 0.f), top);
-        const uint32_t g = (uint32_t)P.occ_grid;
-        const uint32_t cell = ((uint32_t)c2 * g + (uint32_t)c1) * g + (uint32_t)c0;
-        occ = (__ldg(P.canon_bits + (cell >> 5)) >> (cell & 31)) & 1u;
-      }
-      const unsigned word = __ballot_sync(0xffffffffu, occ);
-      if ((threadIdx.x & 31) == 0) reinterpret_cast<uint32_t *>(out)[j >> 5] = word;
+    if (MODE == kModePose && !__any_sync(0xffffffffu, S >= P.occ_smin)) {
+      if (lane == 0) reinterpret_cast<uint32_t *>(out)[tile] = 0u;
       continue;
     }
     if (P.res_enabled) {
-      pos_enc(P, s0, s1, s2, gcol, stride);
-      float r0, r1, r2;
-      residual_f32(P, sW, sB1, gcol, hcol, stride, r0, r1, r2);
-      f0 += r0;
-      f1 += r1;
-      f2 += r2;
+      pos_enc(P, s0, s1, s2, put_g);
+      residual_f32(P, sW, sB1, g, h, o);
+      f0 += o[0];
+      f1 += o[1];
+      f2 += o[2];
     }
-    const bool inside = hash_encode(P, f0, f1, f2, hcol, stride);
-    float o[4];
-    canonical_f32(P, sW, hcol, stride, o);
+    if (MODE == kModePose) {
+      // clamped to the grid as floats before the conversion (fmaxf maps NaN to 0)
+      const float top = (float)(P.occ_grid - 1);
+      const float c0 = fminf(fmaxf(floorf(__fdiv_rn(__fsub_rn(f0, P.bmin[0]), hc[0])), 0.f), top);
+      const float c1 = fminf(fmaxf(floorf(__fdiv_rn(__fsub_rn(f1, P.bmin[1]), hc[1])), 0.f), top);
+      const float c2 = fminf(fmaxf(floorf(__fdiv_rn(__fsub_rn(f2, P.bmin[2]), hc[2])), 0.f), top);
+      const uint32_t gr = (uint32_t)P.occ_grid;
+      const uint32_t cell = ((uint32_t)c2 * gr + (uint32_t)c1) * gr + (uint32_t)c0;
+      const bool occ = S >= P.occ_smin && ((__ldg(P.canon_bits + (cell >> 5)) >> (cell & 31)) & 1u);
+      const unsigned word = __ballot_sync(0xffffffffu, occ);
+      if (lane == 0) reinterpret_cast<uint32_t *>(out)[tile] = word;
+      continue;
+    }
+    const bool inside = hash_encode(P, f0, f1, f2, put_h);
+    canonical_f32(P, sW, h, o);
+    if (!valid) continue;
     const float cr = sigmoidf_(o[0]), cg = sigmoidf_(o[1]), cb = sigmoidf_(o[2]);
     const float sigma = softplusf_(o[3]);
     if (MODE == kModeRender) {
@@ -201,24 +206,30 @@ __global__ void __launch_bounds__(kF32Threads, 1) field_f32_kernel(FieldParams P
   }
 }
 
+// Threads of an FP32 launch: the warps whose activations fit beside the weights (eight with two
+// hidden layers, six with four), and the launch itself.
+static size_t f32_base_smem(const FieldParams &P) { return sizeof(float) * (P.lay.total + kPoseSmem + kWidth); }
+
+template <int MODE>
+static nr_status launch_f32(const FieldParams &P, const float4 *in, uint32_t n_fixed, const uint32_t *n_dev, float *out,
+                            int device, cudaStream_t st) {
+  constexpr size_t kSmemMax = 227 * 1024, kWarpBytes = kF32WarpFloats * sizeof(float);
+  const size_t base = f32_base_smem(P);
+  const int warps = (int)std::min<size_t>(kF32MaxThreads / 32, (kSmemMax - base) / kWarpBytes);
+  const size_t smem = base + warps * kWarpBytes;
+  NR_CHECK_CUDA(cudaFuncSetAttribute(field_f32_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  field_f32_kernel<MODE><<<num_sms(device), 32 * warps, smem, st>>>(P, in, n_fixed, n_dev, out);
+  NR_CHECK_CUDA(cudaGetLastError());
+  return NR_OK;
+}
+
 // Launches the FP32 kernel in kModeDensity or kModePose over P.occ_grid^3 cells,
 // writing occ_grid^3 / 32 words to bits.
 nr_status launch_occupancy_field(const FieldParams &P, int mode, uint32_t *bits, int device, cudaStream_t st) {
-  const size_t smem = field_f32_smem(P);
-  const uint32_t cells = (uint32_t)P.occ_grid * P.occ_grid * P.occ_grid;
-  const int blocks = std::min<int>(num_sms(device), (int)((cells + kF32Threads - 1) / kF32Threads));
-  if (mode == kModeDensity) {
-    NR_CHECK_CUDA(cudaFuncSetAttribute(field_f32_kernel<kModeDensity>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem));
-    field_f32_kernel<kModeDensity><<<blocks, kF32Threads, smem, st>>>(P, nullptr, 0, nullptr,
-                                                                       reinterpret_cast<float *>(bits));
-  } else {
-    NR_CHECK_CUDA(cudaFuncSetAttribute(field_f32_kernel<kModePose>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem));
-    field_f32_kernel<kModePose><<<blocks, kF32Threads, smem, st>>>(P, nullptr, 0, nullptr,
-                                                                    reinterpret_cast<float *>(bits));
-  }
-  NR_CHECK_CUDA(cudaGetLastError());
+  float *words = reinterpret_cast<float *>(bits);
+  const nr_status r = mode == kModeDensity ? launch_f32<kModeDensity>(P, nullptr, 0, nullptr, words, device, st)
+                                           : launch_f32<kModePose>(P, nullptr, 0, nullptr, words, device, st);
+  if (r != NR_OK) return r;
   count_launches(1);
   return NR_OK;
 }
@@ -403,10 +414,6 @@ __global__ void finalize_rays_kernel(const float4 *__restrict__ state, uint32_t 
   out[r] = make_float4(fmaf(c.w, bg0, c.x), fmaf(c.w, bg1, c.y), fmaf(c.w, bg2, c.z), 1.f - c.w);
 }
 
-size_t field_f32_smem(const FieldParams &P) {
-  return sizeof(float) * (P.lay.total + kPoseSmem + kWidth + (size_t)kF32ColRows * kF32Threads);
-}
-
 int num_sms(int device) {
   static int cached[64] = {0};
   if (device < 0 || device >= 64) return 148;
@@ -434,19 +441,8 @@ nr_status launch_field(const FieldParams &P, nr_dtype mlp_dtype, int mode, const
     return NR_EUNSUPPORTED;
   }
   if (mma_path == 3) return launch_field_tf32(P, mode, in, n_fixed, n_dev, out, device, st);
-  const size_t smem = field_f32_smem(P);
-  const int blocks = num_sms(device);
-  if (mode == kModeRender) {
-    NR_CHECK_CUDA(cudaFuncSetAttribute(field_f32_kernel<kModeRender>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem));
-    field_f32_kernel<kModeRender><<<blocks, kF32Threads, smem, st>>>(P, in, n_fixed, n_dev, out);
-  } else {
-    NR_CHECK_CUDA(cudaFuncSetAttribute(field_f32_kernel<kModeQuery>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem));
-    field_f32_kernel<kModeQuery><<<blocks, kF32Threads, smem, st>>>(P, in, n_fixed, n_dev, out);
-  }
-  NR_CHECK_CUDA(cudaGetLastError());
-  return NR_OK;
+  return mode == kModeRender ? launch_f32<kModeRender>(P, in, n_fixed, n_dev, out, device, st)
+                             : launch_f32<kModeQuery>(P, in, n_fixed, n_dev, out, device, st);
 }
 
 // The field kernel a render or query takes (launch_field's mma_path): for bf16/f16 MLPs 0 the
