@@ -3,49 +3,38 @@
 // per step, tf32.cuh) instead of CUDA-core FMAs.
 //
 // Work split: each warp owns a tile of 32 samples.  The gathers (inverse-LBS warp, PE, hash
-// encoding) run one sample per lane in float32 as in the CUDA-core kernel; every layer is a
-// C = W X^T product over the tile (M = outputs, N = the 32 samples, K = inputs) on a padded
-// shared-memory copy of the float32 weights; a sample's activations live in its thread's
-// column of a global scratch buffer (L1/L2 resident), two 64-row buffers used in turn.
+// encoding) run one sample per lane in float32 as in the CUDA-core kernel; every layer reads the
+// tile in shared memory and leaves its output there (frag_fwd).  gamma(x_skel), which layers 1
+// and 4 both see, waits in the warp's image in global memory in between (5 KB, L1/L2 resident).
 #include "field.cuh"
 #include "render.cuh"
 #include "tf32.cuh"
 
 namespace nr {
 
-// rows of a thread's scratch column
-constexpr int kRowGam = 0;                         // gamma(x_skel)
-constexpr int kRowA = kRowGam + kResGammaPad;      // hidden activations, two buffers in turn
-constexpr int kRowB = kRowA + kWidth;
-constexpr int kRowEnc = kRowB + kWidth;            // hash encoding
-constexpr int kRowOut = kRowEnc + kMlpIn;          // the four outputs of either MLP
-static_assert(kRowOut + 4 == kTf32Rows, "scratch rows");
+static_assert(kGamRows == kTf32Rows, "scratch rows");
 
 template <int MODE>
-__global__ void __launch_bounds__(kTf32Threads, 1) field_tf32_kernel(FieldParams P, PadLay PL,
+__global__ void __launch_bounds__(kTf32Threads, 1) field_tf32_kernel(FieldParams P, FragLay W,
                                                                      const float4 *__restrict__ in, uint32_t n_fixed,
                                                                      const uint32_t *__restrict__ n_dev,
                                                                      float *__restrict__ out) {
   extern __shared__ float4 smem4[];
-  float *sW = reinterpret_cast<float *>(smem4);    // the weights in the padded layout PL
-  float *sG = sW + ((PL.total + 3) & ~3);          // pose (and support boxes)
-  float *sB1 = sG + kPoseSmem;                     // residual layer-1 bias with the pose folded in
-  for (int q = 0; q < PL.n_seg; ++q) {
-    const PadSeg &sg = PL.seg[q];
-    for (int i = threadIdx.x; i < sg.rows * sg.cols; i += blockDim.x) {
-      const int rr = i / sg.cols, cc = i - rr * sg.cols;
-      sW[sg.dst + rr * sg.dstride + cc] = __ldg(P.blob + sg.src + i);
-    }
-  }
+  float *sW = reinterpret_cast<float *>(smem4);
+  float *sG = sW + W.total;                        // pose (and support boxes)
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float *xt = sG + kPoseSmem + warp * kTileFloats;
+  stage_frag_weights(P.blob, P.lay, W, P.hidden, sW);
   const float *sBox = stage_pose(P, sG, threadIdx.x, blockDim.x);
-  for (int i = threadIdx.x; i < kWidth; i += blockDim.x) sB1[i] = P.bias1[i];
   __syncthreads();
 
-  const int stride = blockDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float *colbase = P.tf32_scratch + (size_t)blockIdx.x * kTf32Rows * stride;
-  float *col = colbase + threadIdx.x;               // this thread's column
-  float *wcol = colbase + warp * 32;                // the warp's column 0
+  const FragLane L = frag_lane();
   const int warps = blockDim.x >> 5;
+  float *img = P.tf32_scratch + ((size_t)blockIdx.x * warps + warp) * kGamRows * kTileRow;
+  const int eb = (2 * P.L + 7) >> 3;               // blocks of inputs that hold features
+  auto put = [=](int k, float v) {
+    if (k < kGamRows) xt[frag_at(k, lane)] = v;
+  };
   const uint32_t n = n_dev ? *n_dev : n_fixed;
   const uint32_t n_tiles = (n + 31) / 32;
   for (uint32_t tile = blockIdx.x * warps + warp; tile < n_tiles; tile += gridDim.x * warps) {
@@ -69,35 +58,43 @@ __global__ void __launch_bounds__(kTf32Threads, 1) field_tf32_kernel(FieldParams
     float s0, s1, s2, S;
     lbs_warp(P, sG, x0, x1, x2, s0, s1, s2, S, sBox);
     float f0 = s0, f1 = s1, f2 = s2;
+    float c[2][8][4], o[4];
     if (P.res_enabled) {
-      pos_enc(P, s0, s1, s2, col + kRowGam * stride, stride);
+      pos_enc(P, s0, s1, s2, put);
       __syncwarp();
-      warp_fwd<kWidth, kResGammaPad, 0>(sW + PL.r1, kPadRow, wcol, stride, kRowGam, 0, sB1, nullptr, 0, true, kRowA);
-      warp_fwd<kWidth, kWidth, 0>(sW + PL.r2, kPadRow, wcol, stride, kRowA, 0, sW + PL.r2b, nullptr, 0, true, kRowB);
-      warp_fwd<kWidth, kWidth, 0>(sW + PL.r3, kPadRow, wcol, stride, kRowB, 0, sW + PL.r3b, nullptr, 0, true, kRowA);
-      warp_fwd<kWidth, kWidth, kResGammaPad>(sW + PL.r4, kPadRow, wcol, stride, kRowA, kRowGam, sW + PL.r4b, nullptr,
-                                             0, true, kRowB);
-      warp_fwd<4, kWidth, 0>(sW + PL.r5, 4, wcol, stride, kRowB, 0, sW + PL.r5b, nullptr, 0, false, kRowOut);
-      f0 += col[(kRowOut + 0) * stride];
-      f1 += col[(kRowOut + 1) * stride];
-      f2 += col[(kRowOut + 2) * stride];
+      tile_save(xt, img, kGamRows);
+      frag_zero(c);
+      frag_fwd<8>(L, xt, kGamRows / 8, sW + W.r1, kGamRows / 8, 0, c);
+      frag_relu(L, P.bias1, c);
+      frag_store<8>(L, c, xt);
+#pragma unroll 1
+      for (int l = 1; l < 4; ++l) {
+        frag_zero(c);
+        frag_fwd<8>(L, xt, 8, sW + (l == 1 ? W.r2 : l == 2 ? W.r3 : W.r4), l == 3 ? 8 + kGamRows / 8 : 8, 0, c);
+        if (l == 3) {   // layer 4 sees [h3, gamma]
+          tile_load(xt, img, kGamRows);
+          frag_fwd<8>(L, xt, kGamRows / 8, sW + W.r4, 8 + kGamRows / 8, 8, c);
+        }
+        frag_relu(L, sW + (l == 1 ? W.r2b : l == 2 ? W.r3b : W.r4b), c);
+        frag_store<8>(L, c, xt);
+      }
+      frag_out4(L, xt, sW + W.r5, sW + W.r5b, o);
+      f0 += o[0];
+      f1 += o[1];
+      f2 += o[2];
     }
-    const bool inside = hash_encode(P, f0, f1, f2, col + kRowEnc * stride, stride);
+    const bool inside = hash_encode(P, f0, f1, f2, put);
     __syncwarp();
-    warp_fwd<kWidth, kMlpIn, 0>(sW + PL.c0, kPadRow, wcol, stride, kRowEnc, 0, sW + PL.c0b, nullptr, 0, true, kRowA);
-    int cur = kRowA, nxt = kRowB;
-    for (int l = 1; l < P.hidden; ++l) {
-      warp_fwd<kWidth, kWidth, 0>(sW + PL.ch[l - 1], kPadRow, wcol, stride, cur, 0, sW + PL.chb[l - 1], nullptr, 0,
-                                  true, nxt);
-      const int t = cur;
-      cur = nxt;
-      nxt = t;
+#pragma unroll 1
+    for (int l = 0; l < P.hidden; ++l) {
+      frag_zero(c);
+      frag_fwd<8>(L, xt, l ? 8 : eb, sW + (l ? W.ch[l - 1] : W.c0), l ? 8 : kMlpIn / 8, 0, c);
+      frag_relu(L, sW + (l ? W.chb[l - 1] : W.c0b), c);
+      frag_store<8>(L, c, xt);
     }
-    warp_fwd<4, kWidth, 0>(sW + PL.cl, 4, wcol, stride, cur, 0, sW + PL.clb, nullptr, 0, false, kRowOut);
+    frag_out4(L, xt, sW + W.cl, sW + W.clb, o);
     if (valid) {
-      const float o0 = col[kRowOut * stride], o1 = col[(kRowOut + 1) * stride], o2 = col[(kRowOut + 2) * stride],
-                  o3 = col[(kRowOut + 3) * stride];
-      const float cr = sigmoidf_(o0), cg = sigmoidf_(o1), cb = sigmoidf_(o2), sigma = softplusf_(o3);
+      const float cr = sigmoidf_(o[0]), cg = sigmoidf_(o[1]), cb = sigmoidf_(o[2]), sigma = softplusf_(o[3]);
       if (MODE == kModeRender) {
         const float a = inside ? -expm1f(-sigma * delta) * fminf(S, 1.f) : 0.f;
         reinterpret_cast<float4 *>(out)[j] = make_float4(cr, cg, cb, a);
@@ -108,7 +105,6 @@ __global__ void __launch_bounds__(kTf32Threads, 1) field_tf32_kernel(FieldParams
         q[8] = cr; q[9] = cg; q[10] = cb; q[11] = sigma;
       }
     }
-    __syncwarp();   // the next tile reuses the warp's rows
   }
 }
 
@@ -118,17 +114,20 @@ nr_status launch_field_tf32(const FieldParams &P, int mode, const float4 *in, ui
     set_error("the float32 tensor-core tier has no scratch buffer");
     return NR_ESTATE;
   }
-  const PadLay PL = pad_layout(P.lay, P.hidden);
-  const size_t smem = sizeof(float) * (((PL.total + 3) & ~3) + kPoseSmem + kWidth);
+  const FragLay W = frag_layout(P.hidden);
+  // the warps whose tiles fit beside the weights (sixteen with two hidden layers, twelve with four)
+  const size_t base = sizeof(float) * (W.total + kPoseSmem), tile_b = kTileFloats * sizeof(float);
+  const int warps = (int)std::min<size_t>(kTf32Threads / 32, (227 * 1024 - base) / tile_b);
+  const size_t smem = base + warps * tile_b;
   const int blocks = num_sms(device);
   if (mode == kModeRender) {
     NR_CHECK_CUDA(
         cudaFuncSetAttribute(field_tf32_kernel<kModeRender>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    field_tf32_kernel<kModeRender><<<blocks, kTf32Threads, smem, st>>>(P, PL, in, n_fixed, n_dev, out);
+    field_tf32_kernel<kModeRender><<<blocks, 32 * warps, smem, st>>>(P, W, in, n_fixed, n_dev, out);
   } else {
     NR_CHECK_CUDA(
         cudaFuncSetAttribute(field_tf32_kernel<kModeQuery>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    field_tf32_kernel<kModeQuery><<<blocks, kTf32Threads, smem, st>>>(P, PL, in, n_fixed, n_dev, out);
+    field_tf32_kernel<kModeQuery><<<blocks, 32 * warps, smem, st>>>(P, W, in, n_fixed, n_dev, out);
   }
   NR_CHECK_CUDA(cudaGetLastError());
   return NR_OK;

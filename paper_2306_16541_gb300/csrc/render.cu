@@ -478,7 +478,7 @@ nr_status check_field_timeouts(nr_subject *s, cudaStream_t st) {
   return NR_ETIMEOUT;
 }
 
-// One column of kTf32Rows floats per thread of one block per SM (allocated on first use).
+// kTf32Rows floats per thread of one block per SM (allocated on first use).
 static nr_status grow_tf32_scratch(nr_subject *s) {
   const size_t need = (size_t)num_sms(s->device) * kTf32Rows * kTf32Threads;
   if (need <= s->rw_scratch) return NR_OK;

@@ -136,7 +136,7 @@ nr_status launch_field_tc(const FieldParams &P, nr_dtype mlp_dtype, int mode, co
 nr_status fold_frame_biases(nr_subject *s, cudaStream_t st);
 // the float32 tier on the tensor cores: threads per block and scratch rows per thread
 constexpr int kTf32Threads = 512;
-constexpr int kTf32Rows = kResGammaPad + 2 * kWidth + kMlpIn + 4;
+constexpr int kTf32Rows = 40;   // gamma(x_skel), kGamRows
 nr_status launch_field_tf32(const FieldParams &P, int mode, const float4 *in, uint32_t n_fixed, const uint32_t *n_dev,
                             float *out, int device, cudaStream_t st);
 

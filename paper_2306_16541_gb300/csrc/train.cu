@@ -6,23 +6,21 @@
 // refiner's dL/dG) and Adam.
 //
 // Work split:
-//   * the gathers and their adjoints (LBS warp, PE, hash encoding) run one
-//     sample per thread; each thread keeps its sample's activations and deltas
-//     in its own column of a scratch buffer (rows x threads per block);
-//   * both MLPs run per warp of 32 samples on the tensor cores -- forward
-//     layers W X^T, layer backprop W^T D^T, weight gradients D^T H -- as
-//     m16n8k8 TF32 MMAs with three products per step (hi/lo splits) for
-//     float32 accuracy, over a bank-padded shared-memory copy of the weights;
-//   * weight gradients of a warp go into its block's private accumulator
-//     (fire-and-forget atomics shared by the block's warps); one kernel sums
-//     the block accumulators at the end;
-//   * hash-table and weight-volume gradients are scattered with float2 /
-//     float atomics straight into the gradient buffers, warp-aggregated: the
-//     lanes of a run that adds into one cell sum first (run_sum);
-//   * thread slots visit the batch's rays in a scattered order (ray_of), so
-//     that the rays in flight together do not come from one image patch;
-//   * the forward records which slots carry a gradient (live mask); the
-//     backward skips the rest.
+//   * a warp takes 32 samples.  The gathers and their adjoints (LBS warp, PE, hash encoding) run
+//     one sample per lane; the layer at hand -- an activation in the forward, a delta in the
+//     backward -- lies in the warp's shared-memory tile (a row per feature), so both MLPs'
+//     forward and backward layers (m16n8k8 TF32 MMAs, three per step for float32 accuracy) touch
+//     shared memory and registers only.  Every activation that a weight gradient needs goes once
+//     to a per-warp image in global memory, as 16-byte copies of the tile, with the ReLU's sign
+//     bits beside it;
+//   * weight gradients of a warp go into its block's private accumulator, whole MMA fragments
+//     as 16-byte fire-and-forget adds; one kernel sums the block accumulators at the end;
+//   * hash-table and weight-volume gradients are scattered with float2 / float atomics straight
+//     into the gradient buffers, warp-aggregated: the lanes of a run that adds into one cell sum
+//     first (run_sum);
+//   * thread slots visit the batch's rays in a scattered order (ray_of), so that the rays in
+//     flight together do not come from one image patch;
+//   * the forward records which slots carry a gradient (live mask); the backward skips the rest.
 #include <math.h>
 #include <string.h>
 
@@ -32,20 +30,17 @@
 
 namespace nr {
 
-constexpr int kBwdThreads = 384;   // ~160 registers a thread (512 threads at 128 measured slower)
-constexpr int kFwdThreads = 512;   // the forward fits 128, so twice the warps hide its gathers
+constexpr int kTrainThreads = 512;   // at most: sixteen warps of 128 registers
+constexpr size_t kTrainSmem = 227 * 1024;
 
-// Rows of a thread's scratch column (sized for the subject's hidden depth H).
+// Rows (of 32 floats) of a warp's global image, sized for the subject's hidden depth H.
 struct Rows {
-  int gam;     // gamma(x_skel)            48
+  int gam;     // gamma(x_skel)            kGamRows
   int rh;      // residual h1..h4          4 x 64
   int enc;     // hash encoding            32
   int ch;      // canonical h1..hH         H x 64
-  int db;      // two 64-row delta buffers, used in turn by both MLPs' backward
-  int dcl;     // canonical output delta   4
-  int dr5;     // residual output delta    4
-  int denc;    // dL/d encoding            32
-  int dgam;    // dL/d gamma               48
+  int dgam;    // dL/d gamma               kGamRows
+  int sign;    // per hidden layer, a lane's 64 ReLU signs      2 (4 + H)
   int dp;      // dL/d p_i per bone (pose refiner)  3 x 24
   int xs;      // the sample position               3
   int total;
@@ -54,15 +49,12 @@ struct Rows {
 static Rows make_rows(int H) {
   Rows r{};
   int o = 0;
-  r.gam = o; o += kResGammaPad;
+  r.gam = o; o += kGamRows;
   r.rh = o; o += 4 * kWidth;
   r.enc = o; o += kMlpIn;
   r.ch = o; o += H * kWidth;
-  r.db = o; o += 2 * kWidth;
-  r.dcl = o; o += 4;
-  r.dr5 = o; o += 4;
-  r.denc = o; o += kMlpIn;
-  r.dgam = o; o += kResGammaPad;
+  r.dgam = o; o += kGamRows;
+  r.sign = o; o += 2 * (4 + H);
   r.dp = o; o += 3 * kBones;
   r.xs = o; o += 3;
   r.total = o;
@@ -92,7 +84,7 @@ struct TrainDev {
   Rows rw;
   float *dG;              // [F][24][12] dL/dG of every frame (pose refiner), or NULL
   int dG_smem;            // 1: the block sums dG in shared memory first
-  PadLay pl;              // shared-memory layout of the backward kernel's weights
+  FragLay fl;             // shared-memory layout of the weights
   float *pred;            // [n][3] composited colours out, or NULL
   const float *grad_rgb;  // [n][3] dL/dC from the caller, or NULL (MSE against target)
   int forward_only;       // stop after compositing
@@ -254,192 +246,251 @@ __device__ __forceinline__ bool run_sum(uint32_t key_lo, uint32_t key_hi, bool v
 }
 
 // ---------------------------------------------------------------- backward
+// Where the block accumulators hold dW[o][i] of a layer with 64 outputs: the MMA fragments of
+// wgrad64 as they leave the registers, (8-column tile, 16-row tile, lane, value).
+__host__ __device__ __forceinline__ int acc_index(int o, int i) {
+  return (((i >> 3) * 4 + (o >> 4)) * 32 + (o & 7) * 4 + ((i & 7) >> 1)) * 4 + ((o >> 3) & 1) * 2 + (i & 1);
+}
+
 // Warp-level weight gradient of one layer with 64 outputs over the warp's 32 samples,
-// dW[j][k] = sum_s d[s][j] h[s][k], as the product D^T H on the tensor cores
-// (m16n8k8 TF32 MMAs, three per step for float32 accuracy): M = the 64 outputs in four
-// 16-row tiles, K = the 32 samples in four steps of 8, N = the inputs in tiles of 8.  Each
-// finished 16 x 8 tile is added into the block's accumulator acc[wt + k * 64 + j] with
-// fire-and-forget atomics (shared by the block's warps); acc[b + j] += sum_s d[s][j].
-// `wcol` points at the warp's column 0 (row r of sample s is wcol[r * stride + s]).
-__device__ __noinline__ void wgrad64(const float *wcol, int stride, int r_in, int n_in, int r_d, float *acc,
-                                        int wt, int b, bool with_bias) {
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  if (with_bias) {
-    const float4 *p0 = reinterpret_cast<const float4 *>(wcol + (r_d + lane) * stride);
-    const float4 *p1 = reinterpret_cast<const float4 *>(wcol + (r_d + lane + 32) * stride);
+// dW[j][k] = sum_s d[s][j] h[s][k], as the product D^T H on the tensor cores (m16n8k8 TF32 MMAs,
+// three per step for float32 accuracy): M = the 64 outputs in four 16-row tiles, K = the 32
+// samples (taken four consecutive ones a lane, so that a fragment is a 16-byte load; the order of
+// the sum is free), N = the inputs in nb tiles of 8.  D is the shared tile, H the global image of
+// the layer's input.  Each finished 16 x 8 tile is added into the block's accumulator at acc
+// (acc_index) as one 16-byte add per lane; the bias gradient sum_s d[s][j] goes to acc_b[j] and,
+// when given, to acc_f[j].
+__device__ __forceinline__ void wgrad64(const FragLane &L, const float *tile, const float *img, int nb, float *acc,
+                                        float *acc_b, float *acc_f) {
+  const int lane = threadIdx.x & 31;
+  if (acc_b) {
     float s0 = 0.f, s1 = 0.f;
+    const int sw = tile_sw(lane);
+    const float4 *p0 = reinterpret_cast<const float4 *>(tile + lane * kTileRow);
+    const float4 *p1 = reinterpret_cast<const float4 *>(tile + (lane + 32) * kTileRow);
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const float4 a = p0[q], c = p1[q];
+      const float4 a = p0[q ^ sw], c = p1[q ^ sw];
       s0 += (a.x + a.y) + (a.z + a.w);
       s1 += (c.x + c.y) + (c.z + c.w);
     }
-    atomicAdd(acc + b + lane, s0);
-    atomicAdd(acc + b + lane + 32, s1);
+    atomicAdd(acc_b + lane, s0);
+    atomicAdd(acc_b + lane + 32, s1);
+    if (acc_f) {
+      atomicAdd(acc_f + lane, s0);
+      atomicAdd(acc_f + lane + 32, s1);
+    }
   }
-  // A = D^T fragments of two row tiles at a time (one per step of 8 samples), so that the
-  // hi/lo fragments take 64 registers; H is read once per pair of row tiles
+  const int row = L.g * kTileRow;
+  const int at[2] = {row + ((L.t ^ tile_sw(L.g)) << 2), row + (((4 + L.t) ^ tile_sw(L.g)) << 2)};
+  // two row tiles of D at a time, so that their hi/lo fragments take 64 registers; H is read once
+  // per pair
 #pragma unroll 1
   for (int mh = 0; mh < 4; mh += 2) {
     uint32_t ah[2][4][4], al[2][4][4];
 #pragma unroll
-    for (int mm = 0; mm < 2; ++mm) {
-      const float *d0 = wcol + (r_d + 16 * (mh + mm) + g) * stride;
-      const float *d8 = d0 + 8 * stride;
+    for (int m = 0; m < 2; ++m)
 #pragma unroll
-      for (int ks = 0; ks < 4; ++ks) {
-        const int s = 8 * ks + t;
-        tf32_split(d0[s], ah[mm][ks][0], al[mm][ks][0]);
-        tf32_split(d8[s], ah[mm][ks][1], al[mm][ks][1]);
-        tf32_split(d0[s + 4], ah[mm][ks][2], al[mm][ks][2]);
-        tf32_split(d8[s + 4], ah[mm][ks][3], al[mm][ks][3]);
+      for (int j = 0; j < 2; ++j) {
+        const float *d = tile + 16 * (mh + m) * kTileRow + at[j];
+        const float4 u = *reinterpret_cast<const float4 *>(d), v = *reinterpret_cast<const float4 *>(d + 8 * kTileRow);
+        tf32_split(u.x, ah[m][2 * j][0], al[m][2 * j][0]);
+        tf32_split(v.x, ah[m][2 * j][1], al[m][2 * j][1]);
+        tf32_split(u.y, ah[m][2 * j][2], al[m][2 * j][2]);
+        tf32_split(v.y, ah[m][2 * j][3], al[m][2 * j][3]);
+        tf32_split(u.z, ah[m][2 * j + 1][0], al[m][2 * j + 1][0]);
+        tf32_split(v.z, ah[m][2 * j + 1][1], al[m][2 * j + 1][1]);
+        tf32_split(u.w, ah[m][2 * j + 1][2], al[m][2 * j + 1][2]);
+        tf32_split(v.w, ah[m][2 * j + 1][3], al[m][2 * j + 1][3]);
       }
-    }
+    float4 nx0 = *reinterpret_cast<const float4 *>(img + at[0]), nx1 = *reinterpret_cast<const float4 *>(img + at[1]);
 #pragma unroll 1
-    for (int n0 = 0; n0 < n_in; n0 += 8) {
-      uint32_t bh[4][2], bl[4][2];   // B = H fragments of this column tile
-      const float *hk = wcol + (r_in + n0 + g) * stride;
+    for (int n = 0; n < nb; ++n) {
+      const float hv[8] = {nx0.x, nx0.y, nx0.z, nx0.w, nx1.x, nx1.y, nx1.z, nx1.w};
+      if (n + 1 < nb) {   // the next tile's loads run under this one's products
+        const float *h = img + (n + 1) * 8 * kTileRow;
+        nx0 = *reinterpret_cast<const float4 *>(h + at[0]);
+        nx1 = *reinterpret_cast<const float4 *>(h + at[1]);
+      }
+      float c[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
       for (int ks = 0; ks < 4; ++ks) {
-        tf32_split(hk[8 * ks + t], bh[ks][0], bl[ks][0]);
-        tf32_split(hk[8 * ks + t + 4], bh[ks][1], bl[ks][1]);
+        uint32_t bh[2], bl[2];
+        tf32_split(hv[2 * ks], bh[0], bl[0]);
+        tf32_split(hv[2 * ks + 1], bh[1], bl[1]);
+#pragma unroll
+        for (int m = 0; m < 2; ++m) mma_tf32(c[m], al[m][ks], bh);
+#pragma unroll
+        for (int m = 0; m < 2; ++m) mma_tf32(c[m], ah[m][ks], bl);
+#pragma unroll
+        for (int m = 0; m < 2; ++m) mma_tf32(c[m], ah[m][ks], bh);
       }
 #pragma unroll
-      for (int mm = 0; mm < 2; ++mm) {
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-          mma_tf32(c, al[mm][ks], bh[ks]);
-          mma_tf32(c, ah[mm][ks], bl[ks]);
-          mma_tf32(c, ah[mm][ks], bh[ks]);
-        }
-        // c = C[16m + g][n0 + 2t], C[16m + g][n0 + 2t + 1], C[16m + g + 8][n0 + 2t], C[16m + g + 8][n0 + 2t + 1]
-        float *o = acc + wt + (n0 + 2 * t) * kWidth + 16 * (mh + mm) + g;
-        atomicAdd(o, c[0]);
-        atomicAdd(o + kWidth, c[1]);
-        atomicAdd(o + 8, c[2]);
-        atomicAdd(o + kWidth + 8, c[3]);
-      }
+      for (int m = 0; m < 2; ++m)
+        atomicAdd(reinterpret_cast<float4 *>(acc) + (n * 4 + mh + m) * 32 + lane,
+                  make_float4(c[m][0], c[m][1], c[m][2], c[m][3]));
     }
   }
 }
 
-// Same for a layer with 4 (padded) outputs and 64 inputs: lane owns input rows k = lane, lane + 32.
-__device__ __forceinline__ void wgrad4(const float *wcol, int stride, int r_in, int r_d, int n_out, float *acc, int wt,
-                                       int b) {
-  const int lane = threadIdx.x & 31;
+// Same for a layer with n_out <= 4 outputs and 64 inputs: lane owns input rows k = lane, lane + 32
+// of the image, the deltas are the tile's rows 0..n_out-1.
+__device__ __forceinline__ void wgrad4(const float *tile, const float *img, int n_out, float *acc, float *acc_b) {
+  const int lane = threadIdx.x & 31, sw = tile_sw(lane);
   float h0[32], h1[32];
-  const float4 *p0 = reinterpret_cast<const float4 *>(wcol + (r_in + lane) * stride);
-  const float4 *p1 = reinterpret_cast<const float4 *>(wcol + (r_in + lane + 32) * stride);
+  const float4 *p0 = reinterpret_cast<const float4 *>(img + lane * kTileRow);
+  const float4 *p1 = reinterpret_cast<const float4 *>(img + (lane + 32) * kTileRow);
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const float4 a = p0[q], c = p1[q];
+    const float4 a = p0[q ^ sw], c = p1[q ^ sw];
     h0[4 * q] = a.x; h0[4 * q + 1] = a.y; h0[4 * q + 2] = a.z; h0[4 * q + 3] = a.w;
     h1[4 * q] = c.x; h1[4 * q + 1] = c.y; h1[4 * q + 2] = c.z; h1[4 * q + 3] = c.w;
   }
+#pragma unroll 1
   for (int j = 0; j < n_out; ++j) {
-    const float4 *pd = reinterpret_cast<const float4 *>(wcol + (r_d + j) * stride);
+    const float4 *pd = reinterpret_cast<const float4 *>(tile + j * kTileRow);
+    const int swj = tile_sw(j);
     float a0 = 0.f, a1 = 0.f, sb = 0.f;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const float4 d = pd[q];
+      const float4 d = pd[q ^ swj];
       a0 = fmaf(h0[4 * q], d.x, fmaf(h0[4 * q + 1], d.y, fmaf(h0[4 * q + 2], d.z, fmaf(h0[4 * q + 3], d.w, a0))));
       a1 = fmaf(h1[4 * q], d.x, fmaf(h1[4 * q + 1], d.y, fmaf(h1[4 * q + 2], d.z, fmaf(h1[4 * q + 3], d.w, a1))));
       sb += d.x + d.y + d.z + d.w;
     }
-    atomicAdd(acc + wt + lane * 4 + j, a0);
-    atomicAdd(acc + wt + (lane + 32) * 4 + j, a1);
-    if (lane == 0) atomicAdd(acc + b + j, sb);
+    atomicAdd(acc + lane * 4 + j, a0);
+    atomicAdd(acc + (lane + 32) * 4 + j, a1);
+    if (lane == 0) atomicAdd(acc_b + j, sb);
   }
 }
 
-// The backward of one layer for the warp's 32 samples on the tensor cores:
-//   out[s][i] = (sum_o W^T[i][o] delta[s][o]) * (h[s][i] > 0)     (no mask when r_h < 0)
-// as C = W^T D^T with M = IN (16-row tiles of inputs), N = the 32 samples (4 tiles of 8),
-// K = OUT (steps of 8; a 4-output layer pads its step with zeros); m16n8k8 TF32 MMAs, three
-// per step for float32 accuracy.  W^T comes from the padded shared copy (row i at Wt + i * rs),
-// delta from scratch rows r_d.., the mask from rows r_h..; the result goes to rows r_out..
-// (added to them when `accumulate`).  Every lane of the warp must take part.
-template <int OUT, int IN>
-__device__ __noinline__ void warp_back(const float *__restrict__ Wt, int rs, float *wcol, int stride, int r_d,
-                                          int r_h, int r_out, bool accumulate) {
-  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  constexpr int KS = (OUT + 7) / 8, MT = IN / 16;
-  float acc[MT][4][4];
+// ------------------------------------------------------------ the forward of a tile
+// A finished hidden layer: into the tile and, when the backward follows, its image and signs.
+template <bool SAVE>
+__device__ __forceinline__ void layer_done(const FragLane &L, const float (&c)[2][8][4], float *tile, float *img,
+                                           float *sign) {
+  frag_store<8>(L, c, tile);
+  if (!SAVE) return;
+  tile_save(tile, img, kWidth);
+  uint32_t bits[2] = {0u, 0u};
 #pragma unroll
-  for (int m = 0; m < MT; ++m)
+  for (int m = 0; m < 2; ++m)
 #pragma unroll
-    for (int n = 0; n < 4; ++n)
+    for (int n = 0; n < 8; ++n)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) acc[m][n][q] = 0.f;
-#pragma unroll 1
-  for (int ks = 0; ks < KS; ++ks) {
-    const int o0 = 8 * ks + t, o1 = o0 + 4;
-    uint32_t bh[4][2], bl[4][2];
+      for (int q = 0; q < 4; ++q) bits[m] |= (c[m][n][q] > 0.f ? 1u : 0u) << (4 * n + q);
+  reinterpret_cast<uint2 *>(sign)[threadIdx.x & 31] = make_uint2(bits[0], bits[1]);
+}
+
+// The backward's counterpart: the delta of the layer below, through its ReLU, into the tile.
+__device__ __forceinline__ void delta_done(const FragLane &L, uint2 sign, float (&c)[2][8][4], float *tile) {
 #pragma unroll
-    for (int n = 0; n < 4; ++n) {
-      const float u0 = o0 < OUT ? wcol[(r_d + o0) * stride + 8 * n + g] : 0.f;
-      const float u1 = o1 < OUT ? wcol[(r_d + o1) * stride + 8 * n + g] : 0.f;
-      tf32_split(u0, bh[n][0], bl[n][0]);
-      tf32_split(u1, bh[n][1], bl[n][1]);
-    }
+  for (int m = 0; m < 2; ++m)
 #pragma unroll
-    for (int m = 0; m < MT; ++m) {
-      const float *w0 = Wt + (16 * m + g) * rs, *w8 = w0 + 8 * rs;
-      uint32_t ah[4], al[4];
-      tf32_split(o0 < OUT ? w0[o0] : 0.f, ah[0], al[0]);
-      tf32_split(o0 < OUT ? w8[o0] : 0.f, ah[1], al[1]);
-      tf32_split(o1 < OUT ? w0[o1] : 0.f, ah[2], al[2]);
-      tf32_split(o1 < OUT ? w8[o1] : 0.f, ah[3], al[3]);
+    for (int n = 0; n < 8; ++n)
 #pragma unroll
-      for (int n = 0; n < 4; ++n) {
-        mma_tf32(acc[m][n], al, bh[n]);
-        mma_tf32(acc[m][n], ah, bl[n]);
-        mma_tf32(acc[m][n], ah, bh[n]);
-      }
-    }
+      for (int q = 0; q < 4; ++q)
+        if (!(((m ? sign.y : sign.x) >> (4 * n + q)) & 1u)) c[m][n][q] = 0.f;
+  frag_store<8>(L, c, tile);
+}
+
+// One lane's sample through the field: its warped point, its canonical point, the four raw
+// outputs and whether the canonical point lies in the box.
+struct FieldOut {
+  float xs0, xs1, xs2, S, xf0, xf1, xf2, o[4];
+  bool inside;
+};
+
+// Both MLPs of the warp's tile for the 32 samples at s (lanes without a sample: zeros), the pose
+// being training frame f's.  SAVE: activations, encodings and signs go to the image for the
+// backward.  Every lane of the warp must take part.  Not inlined: compiled by itself, the forward
+// gets the same fused multiply-adds in every kernel that calls it, so the colours of a step are
+// those of the forward-only call bit for bit (inlined into the backward they differed in the last
+// bit, and with them the side of a kink that a few samples fall on).
+template <bool SAVE>
+__device__ __noinline__ void field_forward(const FieldParams &P, const TrainDev &T, const FragLane &L,
+                                              const float *sW, float *tile, float *img, const float4 s, bool active,
+                                              uint32_t f, FieldOut &F) {
+  const FragLay &W = T.fl;
+  const Rows &R = T.rw;
+  const int lane = threadIdx.x & 31;
+  auto put = [=](int k, float v) {
+    if (k < kGamRows) tile[frag_at(k, lane)] = v;
+  };
+  F.xs0 = F.xs1 = F.xs2 = F.S = 0.f;
+  if (active) {
+    lbs_warp(P, T.fG + (size_t)f * kBones * 12, s.x, s.y, s.z, F.xs0, F.xs1, F.xs2, F.S);
+    if (P.res_enabled) pos_enc(P, F.xs0, F.xs1, F.xs2, put);
+  } else if (P.res_enabled) {
+    for (int q = 0; q < kGamRows; ++q) put(q, 0.f);
   }
-  // acc[m][n] = C[16m + g][8n + 2t], C[16m + g][8n + 2t + 1], C[16m + g + 8][8n + 2t], C[16m + g + 8][8n + 2t + 1]
-#pragma unroll
-  for (int m = 0; m < MT; ++m)
-#pragma unroll
-    for (int n = 0; n < 4; ++n)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = 16 * m + g + (q >= 2 ? 8 : 0), smp = 8 * n + 2 * t + (q & 1);
-        float v = acc[m][n][q];
-        if (r_h >= 0 && !(wcol[(r_h + i) * stride + smp] > 0.f)) v = 0.f;
-        float *dst = wcol + (r_out + i) * stride + smp;
-        *dst = accumulate ? *dst + v : v;
+  F.xf0 = F.xs0;
+  F.xf1 = F.xs1;
+  F.xf2 = F.xs2;
+  float c[2][8][4];
+  auto sign_of = [&](int l) { return img + (R.sign + 2 * l) * kTileRow; };
+  if (P.res_enabled) {
+    __syncwarp();
+    tile_save(tile, img + R.gam * kTileRow, kGamRows);
+    frag_zero(c);
+    frag_fwd<8>(L, tile, kGamRows / 8, sW + W.r1, kGamRows / 8, 0, c);
+    frag_relu_rows(L, T.fbias1, (int)f, c);
+    layer_done<SAVE>(L, c, tile, img + R.rh * kTileRow, sign_of(0));
+#pragma unroll 1
+    for (int l = 1; l < 4; ++l) {
+      frag_zero(c);
+      frag_fwd<8>(L, tile, 8, sW + (l == 1 ? W.r2 : l == 2 ? W.r3 : W.r4), l == 3 ? 8 + kGamRows / 8 : 8, 0, c);
+      if (l == 3) {   // layer 4 sees [h3, gamma]
+        tile_load(tile, img + R.gam * kTileRow, kGamRows);
+        frag_fwd<8>(L, tile, kGamRows / 8, sW + W.r4, 8 + kGamRows / 8, 8, c);
       }
-  __syncwarp();   // the next layer reads these rows through other lanes
+      frag_relu(L, sW + (l == 1 ? W.r2b : l == 2 ? W.r3b : W.r4b), c);
+      layer_done<SAVE>(L, c, tile, img + (R.rh + l * kWidth) * kTileRow, sign_of(l));
+    }
+    float xr[4];
+    frag_out4(L, tile, sW + W.r5, sW + W.r5b, xr);
+    F.xf0 += xr[0];
+    F.xf1 += xr[1];
+    F.xf2 += xr[2];
+  }
+  F.inside = false;
+  auto put_enc = [=](int k, float v) { tile[frag_at(k, lane)] = v; };
+  if (active) {
+    F.inside = hash_encode(P, F.xf0, F.xf1, F.xf2, put_enc);
+  } else {
+    for (int q = 0; q < kMlpIn; ++q) put_enc(q, 0.f);
+  }
+  __syncwarp();
+  const int eb = (2 * P.L + 7) >> 3;   // blocks of inputs that hold features
+  if (SAVE) tile_save(tile, img + R.enc * kTileRow, 8 * eb);
+#pragma unroll 1
+  for (int l = 0; l < P.hidden; ++l) {
+    frag_zero(c);
+    frag_fwd<8>(L, tile, l ? 8 : eb, sW + (l ? W.ch[l - 1] : W.c0), l ? 8 : kMlpIn / 8, 0, c);
+    frag_relu(L, sW + (l ? W.chb[l - 1] : W.c0b), c);
+    layer_done<SAVE>(L, c, tile, img + (R.ch + l * kWidth) * kTileRow, sign_of(4 + l));
+  }
+  frag_out4(L, tile, sW + W.cl, sW + W.clb, F.o);
+}
+
+// A slot's (r, g, b, alpha).
+__device__ __forceinline__ float4 slot_colour(const FieldOut &F, float delta) {
+  const float a = F.inside ? -expm1f(-softplusf_(F.o[3]) * delta) * fminf(F.S, 1.f) : 0.f;
+  return make_float4(sigmoidf_(F.o[0]), sigmoidf_(F.o[1]), sigmoidf_(F.o[2]), a);
 }
 
 // ------------------------------------------------------------ forward field
-// The float32 field with the pose of each sample's frame, laid out like the backward
-// kernel: per-sample gathers (LBS warp, PE, hash encoding) one sample per thread, both MLPs
-// as warp-level tensor-core layers over the samples' scratch columns (float32 accuracy).
-// Writes (r, g, b, alpha) per sample slot (zero for a ray that misses the box).
-__global__ void __launch_bounds__(kFwdThreads, 1) train_fwd_kernel(FieldParams P, TrainDev T) {
+// The float32 field with the pose of each sample's frame.  Writes (r, g, b, alpha) per sample
+// slot (zero for a ray that misses the box).
+__global__ void __launch_bounds__(kTrainThreads, 1) train_fwd_kernel(FieldParams P, TrainDev T) {
   extern __shared__ float4 smem4[];
-  float *sW = reinterpret_cast<float *>(smem4);        // the weights in the padded layout T.pl
-  for (int q = 0; q < T.pl.n_seg; ++q) {
-    const PadSeg &sg = T.pl.seg[q];
-    for (int i = threadIdx.x; i < sg.rows * sg.cols; i += blockDim.x) {
-      const int rr = i / sg.cols, cc = i - rr * sg.cols;
-      sW[sg.dst + rr * sg.dstride + cc] = __ldg(P.blob + sg.src + i);
-    }
-  }
+  float *sW = reinterpret_cast<float *>(smem4);
+  const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  float *tile = sW + T.fl.total + warp * kTileFloats;
+  stage_frag_weights(P.blob, P.lay, T.fl, P.hidden, sW);
   __syncthreads();
-  const PadLay &PL = T.pl;
-  const int stride = blockDim.x;
-  const int warp = threadIdx.x >> 5;
-  const Rows &RW = T.rw;
-  const int R_GAM = RW.gam, R_RH = RW.rh, R_ENC = RW.enc, R_CH = RW.ch, D_CL = RW.dcl, D_R5 = RW.dr5;
-  float *colbase = T.scratch + (size_t)blockIdx.x * RW.total * stride;
-  float *col = colbase + threadIdx.x;
-  float *wcol = colbase + warp * 32;
-  const int H = P.hidden;
+  const FragLane L = frag_lane();
+  float *img = T.scratch + ((size_t)blockIdx.x * warps + warp) * T.rw.total * kTileRow;
   const uint32_t n = T.n_rays * T.S;
   const uint32_t step = gridDim.x * blockDim.x;
   const uint32_t n_iter = (n + step - 1) / step;
@@ -454,91 +505,52 @@ __global__ void __launch_bounds__(kFwdThreads, 1) train_fwd_kernel(FieldParams P
       continue;
     }
     const uint32_t f = active ? T.frame_id[r] : 0;
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    float S = 0.f, f0 = 0.f, f1 = 0.f, f2 = 0.f;
-    if (active) {
-      s = T.samp[j];
-      float s0, s1, s2;
-      lbs_warp(P, T.fG + (size_t)f * kBones * 12, s.x, s.y, s.z, s0, s1, s2, S);
-      f0 = s0;
-      f1 = s1;
-      f2 = s2;
-      pos_enc(P, s0, s1, s2, col + R_GAM * stride, stride);
-    } else {
-      for (int q = 0; q < kResGammaPad; ++q) col[(R_GAM + q) * stride] = 0.f;
-    }
-    __syncwarp();
-    if (P.res_enabled) {
-      warp_fwd<kWidth, kResGammaPad, 0>(sW + PL.r1, kPadRow, wcol, stride, R_GAM, 0, nullptr, T.fbias1, (int)f,
-                                        true, R_RH + 0 * kWidth);
-      warp_fwd<kWidth, kWidth, 0>(sW + PL.r2, kPadRow, wcol, stride, R_RH + 0 * kWidth, 0, sW + PL.r2b, nullptr, 0,
-                                  true, R_RH + 1 * kWidth);
-      warp_fwd<kWidth, kWidth, 0>(sW + PL.r3, kPadRow, wcol, stride, R_RH + 1 * kWidth, 0, sW + PL.r3b, nullptr, 0,
-                                  true, R_RH + 2 * kWidth);
-      warp_fwd<kWidth, kWidth, kResGammaPad>(sW + PL.r4, kPadRow, wcol, stride, R_RH + 2 * kWidth, R_GAM, sW + PL.r4b,
-                                             nullptr, 0, true, R_RH + 3 * kWidth);
-      warp_fwd<4, kWidth, 0>(sW + PL.r5, 4, wcol, stride, R_RH + 3 * kWidth, 0, sW + PL.r5b, nullptr, 0, false, D_R5);
-    }
-    bool inside = false;
-    if (active) {
-      if (P.res_enabled) {
-        f0 += col[(D_R5 + 0) * stride];
-        f1 += col[(D_R5 + 1) * stride];
-        f2 += col[(D_R5 + 2) * stride];
-      }
-      inside = hash_encode(P, f0, f1, f2, col + R_ENC * stride, stride);
-    } else {
-      for (int q = 0; q < kMlpIn; ++q) col[(R_ENC + q) * stride] = 0.f;
-    }
-    __syncwarp();
-    warp_fwd<kWidth, kMlpIn, 0>(sW + PL.c0, kPadRow, wcol, stride, R_ENC, 0, sW + PL.c0b, nullptr, 0, true, R_CH);
-    for (int l = 1; l < H; ++l)
-      warp_fwd<kWidth, kWidth, 0>(sW + PL.ch[l - 1], kPadRow, wcol, stride, R_CH + (l - 1) * kWidth, 0,
-                                  sW + PL.chb[l - 1], nullptr, 0, true, R_CH + l * kWidth);
-    warp_fwd<4, kWidth, 0>(sW + PL.cl, 4, wcol, stride, R_CH + (H - 1) * kWidth, 0, sW + PL.clb, nullptr, 0, false,
-                           D_CL);
+    const float4 s = active ? T.samp[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+    FieldOut F;
+    field_forward<false>(P, T, L, sW, tile, img, s, active, f, F);
     {
       // the slots whose samples carry a gradient (in the box, warped into the canonical box);
       // the backward skips the others, which add exactly zero
-      const uint32_t lw = __ballot_sync(0xffffffffu, active && inside);
+      const uint32_t lw = __ballot_sync(0xffffffffu, active && F.inside);
       if ((threadIdx.x & 31) == 0 && q < n) T.live[q >> 5] = lw;
     }
-    if (q < n) {
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (active) {
-        const float o0 = col[D_CL * stride], o1 = col[(D_CL + 1) * stride], o2 = col[(D_CL + 2) * stride],
-                    o3 = col[(D_CL + 3) * stride];
-        const float a = inside ? -expm1f(-softplusf_(o3) * s.w) * fminf(S, 1.f) : 0.f;
-        v = make_float4(sigmoidf_(o0), sigmoidf_(o1), sigmoidf_(o2), a);
-      }
-      T.out[j] = v;
-    }
+    if (q < n) T.out[j] = active ? slot_colour(F, s.w) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
 }
 
 // The compositing adjoint of train_composite_kernel for the RB rays whose slots a block holds
-// (ray slots rs0 .. rs0 + RB - 1; local ray lr's samples at o[lr S ..]), by the block's first
-// warp: o[] holds each slot's (r, g, b, alpha) on entry and its (dL/dc, dL/dalpha) on exit,
-// Ts[] the transmittance in front of each sample.  Same arithmetic in the same order.
-__device__ __forceinline__ void composite_rays(const TrainDev &T, float4 *o, float *Ts, uint32_t rs0, uint32_t RB) {
+// (ray slots rs0 .. rs0 + RB - 1; local ray lr's samples are the block's slots lr S ..), by the
+// block's first warp.  Slot i's (r, g, b, alpha) lies in its warp's tile, at slot_at(i), on entry
+// and its (dL/dc, dL/dalpha) on exit; the transmittance in front of it goes 128 floats behind.
+// Same arithmetic in the same order, the slots loaded eight ahead of the chain.
+__device__ __forceinline__ int slot_at(uint32_t i) { return (int)(i >> 5) * kTileFloats + (int)(i & 31) * 4; }
+__device__ __forceinline__ int slot_T(uint32_t i) { return (int)(i >> 5) * kTileFloats + 128 + (int)(i & 31); }
+
+__device__ __forceinline__ void composite_rays(const TrainDev &T, float *tiles, uint32_t rs0, uint32_t RB) {
   const int lane = threadIdx.x & 31;
   float lsum = 0.f;
   for (uint32_t lr = lane; lr < RB; lr += 32) {
     const uint32_t rs = rs0 + lr;
     if (rs >= T.n_rays) break;
     const uint32_t r = (uint32_t)(((uint64_t)rs * T.ray_mul) % T.n_rays);
-    float4 *v4 = o + (size_t)lr * T.S;
-    float *t4 = Ts + (size_t)lr * T.S;
+    const uint32_t i0 = lr * T.S;
     const uint32_t cnt = T.raycnt[r];
     float Tr = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
-    for (uint32_t i = 0; i < cnt; ++i) {
-      const float4 v = v4[i];
-      t4[i] = Tr;
-      const float w = Tr * v.w;
-      c0 = fmaf(w, v.x, c0);
-      c1 = fmaf(w, v.y, c1);
-      c2 = fmaf(w, v.z, c2);
-      Tr *= 1.f - v.w;
+    for (uint32_t i = 0; i < cnt; i += 8) {
+      float4 v[8];
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k)
+        if (i + k < cnt) v[k] = *reinterpret_cast<const float4 *>(tiles + slot_at(i0 + i + k));
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k) {
+        if (i + k >= cnt) break;
+        tiles[slot_T(i0 + i + k)] = Tr;
+        const float w = Tr * v[k].w;
+        c0 = fmaf(w, v[k].x, c0);
+        c1 = fmaf(w, v[k].y, c1);
+        c2 = fmaf(w, v[k].z, c2);
+        Tr *= 1.f - v[k].w;
+      }
     }
     const float C0 = fmaf(Tr, T.bg[0], c0), C1 = fmaf(Tr, T.bg[1], c1), C2 = fmaf(Tr, T.bg[2], c2);
     if (T.pred) {
@@ -560,13 +572,26 @@ __device__ __forceinline__ void composite_rays(const TrainDev &T, float4 *o, flo
       g2 = scale * e2;
     }
     float B = T.bg[0] * g0 + T.bg[1] * g1 + T.bg[2] * g2;
-    for (int i = (int)cnt - 1; i >= 0; --i) {
-      const float4 v = v4[i];
-      const float Ti = t4[i];
-      const float cg = v.x * g0 + v.y * g1 + v.z * g2;
-      const float ta = Ti * v.w;
-      v4[i] = make_float4(ta * g0, ta * g1, ta * g2, Ti * (cg - B));
-      B = fmaf(v.w, cg, (1.f - v.w) * B);
+    for (uint32_t e = cnt; e > 0;) {   // samples e - 1, e - 2, ..: eight at a time
+      const uint32_t m = e < 8u ? e : 8u;
+      float4 v[8];
+      float t[8];
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k)
+        if (k < m) {
+          v[k] = *reinterpret_cast<const float4 *>(tiles + slot_at(i0 + e - 1 - k));
+          t[k] = tiles[slot_T(i0 + e - 1 - k)];
+        }
+#pragma unroll
+      for (uint32_t k = 0; k < 8; ++k) {
+        if (k >= m) break;
+        const float cg = v[k].x * g0 + v[k].y * g1 + v[k].z * g2;
+        const float ta = t[k] * v[k].w;
+        *reinterpret_cast<float4 *>(tiles + slot_at(i0 + e - 1 - k)) =
+            make_float4(ta * g0, ta * g1, ta * g2, t[k] * (cg - B));
+        B = fmaf(v[k].w, cg, (1.f - v[k].w) * B);
+      }
+      e -= m;
     }
   }
 #pragma unroll
@@ -574,40 +599,28 @@ __device__ __forceinline__ void composite_rays(const TrainDev &T, float4 *o, flo
   if (lane == 0 && lsum != 0.f) atomicAdd(T.loss, lsum / (3.f * (float)T.n_rays));
 }
 
-// One thread per sample: forward recompute (activations into the thread's scratch
-// column), backward, scatter-adds, then the warp's weight-gradient reduction.
-// FUSED: the forward and the compositing adjoint run here too, so that neither train_fwd_kernel
-// nor train_composite_kernel is needed: the block takes groups of whole rays (RB = blockDim / S
-// of them), evaluates every sample once, composites its rays in shared memory and goes straight
-// on to the backward with the activations still in its columns.
+// A warp per 32 samples: forward (activations to the warp's image), backward, scatter-adds and the
+// warp's weight gradients.
+// FUSED: the block takes groups of whole rays (RB = blockDim / S of them), evaluates every sample
+// once, composites its rays in shared memory and goes straight on to the backward, so that neither
+// train_fwd_kernel nor train_composite_kernel is needed.
 template <bool FUSED>
-__global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P, TrainDev T) {
+__global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams P, TrainDev T) {
   extern __shared__ float4 smem4[];
-  float *sW = reinterpret_cast<float *>(smem4);        // the weights in the padded layout T.pl
-  float *sdG = sW + T.pl.total;                        // [F][24][12] when T.dG_smem
-  // FUSED: each slot's (r, g, b, alpha), then its adjoint [SB], and transmittances [SB]
-  float4 *sOut = reinterpret_cast<float4 *>(sdG + (T.dG && T.dG_smem ? T.n_frames * kBones * 12 : 0));
-  float *sT = reinterpret_cast<float *>(sOut + blockDim.x);
-  for (int q = 0; q < T.pl.n_seg; ++q) {
-    const PadSeg &sg = T.pl.seg[q];
-    for (int i = threadIdx.x; i < sg.rows * sg.cols; i += blockDim.x) {
-      const int rr = i / sg.cols, cc = i - rr * sg.cols;
-      sW[sg.dst + rr * sg.dstride + cc] = __ldg(P.blob + sg.src + i);
-    }
-  }
+  float *sW = reinterpret_cast<float *>(smem4);
+  float *tiles = sW + T.fl.total;                      // a tile per warp
+  float *sdG = tiles + (blockDim.x >> 5) * kTileFloats;   // [F][24][12] when T.dG_smem
+  stage_frag_weights(P.blob, P.lay, T.fl, P.hidden, sW);
   if (T.dG && T.dG_smem)
     for (int i = threadIdx.x; i < T.n_frames * kBones * 12; i += blockDim.x) sdG[i] = 0.f;
   __syncthreads();
   const BlobLayout &Ly = P.lay;                        // the gradient accumulators' layout
-  const PadLay &PL = T.pl;
-  const int stride = blockDim.x;
+  const FragLay &W = T.fl;
+  const Rows &R = T.rw;
+  const FragLane L = frag_lane();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const Rows &RW = T.rw;
-  const int R_GAM = RW.gam, R_RH = RW.rh, R_ENC = RW.enc, R_CH = RW.ch, D_B = RW.db, D_CL = RW.dcl, D_R5 = RW.dr5,
-            R_DENC = RW.denc, R_DGAM = RW.dgam, R_DP = RW.dp, R_XS = RW.xs, kRows = RW.total;
-  float *colbase = T.scratch + (size_t)blockIdx.x * kRows * stride;
-  float *col = colbase + threadIdx.x;                  // this thread's column
-  float *wcol = colbase + warp * 32;                   // the warp's column 0
+  float *tile = tiles + warp * kTileFloats;
+  float *img = T.scratch + ((size_t)blockIdx.x * (blockDim.x >> 5) + warp) * R.total * kTileRow;
   float *acc = T.wacc + (size_t)blockIdx.x * T.acc_floats;
   float *accF = acc + Ly.total;                        // per-frame first-layer bias gradients [F][64]
   const int H = P.hidden;
@@ -635,121 +648,75 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P
     float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
     if (!FUSED && active) g4 = __ldcs(T.out + j);
     const bool run = !FUSED || __any_sync(0xffffffffu, active);   // warp-uniform
-    // per-sample state carried across the warp-level phases below
-    const float *G = T.fG + (size_t)f * kBones * 12;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    float xs0 = 0.f, xs1 = 0.f, xs2 = 0.f, S = 0.f, xf0 = 0.f, xf1 = 0.f, xf2 = 0.f, dS_alpha = 0.f;
-    bool inside = false;
+    FieldOut F{};
     if (run) {
-    // ---------------- forward recompute: per-sample gathers, warp-level MLP layers
-    if (active) {
-      s = __ldcs(T.samp + j);
-      lbs_warp(P, G, s.x, s.y, s.z, xs0, xs1, xs2, S);
-      xf0 = xs0;
-      xf1 = xs1;
-      xf2 = xs2;
-      pos_enc(P, xs0, xs1, xs2, col + R_GAM * stride, stride);
-    } else {
-      for (int q = 0; q < kResGammaPad; ++q) col[(R_GAM + q) * stride] = 0.f;
-    }
-    __syncwarp();
-    if (P.res_enabled) {
-      warp_fwd<kWidth, kResGammaPad, 0>(sW + PL.r1, kPadRow, wcol, stride, R_GAM, 0, nullptr, T.fbias1, (int)f,
-                                        true, R_RH + 0 * kWidth);
-      warp_fwd<kWidth, kWidth, 0>(sW + PL.r2, kPadRow, wcol, stride, R_RH + 0 * kWidth, 0, sW + PL.r2b, nullptr, 0,
-                                  true, R_RH + 1 * kWidth);
-      warp_fwd<kWidth, kWidth, 0>(sW + PL.r3, kPadRow, wcol, stride, R_RH + 1 * kWidth, 0, sW + PL.r3b, nullptr, 0,
-                                  true, R_RH + 2 * kWidth);
-      warp_fwd<kWidth, kWidth, kResGammaPad>(sW + PL.r4, kPadRow, wcol, stride, R_RH + 2 * kWidth, R_GAM, sW + PL.r4b,
-                                             nullptr, 0, true, R_RH + 3 * kWidth);
-      // x_res into the (not yet used) rows of the residual output's delta
-      warp_fwd<4, kWidth, 0>(sW + PL.r5, 4, wcol, stride, R_RH + 3 * kWidth, 0, sW + PL.r5b, nullptr, 0, false, D_R5);
-    }
-    if (active) {
-      if (P.res_enabled) {
-        xf0 += col[(D_R5 + 0) * stride];
-        xf1 += col[(D_R5 + 1) * stride];
-        xf2 += col[(D_R5 + 2) * stride];
-      } else {
-        for (int q = 0; q < 4 * kWidth; ++q) col[(R_RH + q) * stride] = 0.f;
-      }
-      inside = hash_encode(P, xf0, xf1, xf2, col + R_ENC * stride, stride);
-    } else {
-      for (int q = 0; q < kMlpIn; ++q) col[(R_ENC + q) * stride] = 0.f;
-    }
-    __syncwarp();
-    warp_fwd<kWidth, kMlpIn, 0>(sW + PL.c0, kPadRow, wcol, stride, R_ENC, 0, sW + PL.c0b, nullptr, 0, true, R_CH);
-    for (int l = 1; l < H; ++l)
-      warp_fwd<kWidth, kWidth, 0>(sW + PL.ch[l - 1], kPadRow, wcol, stride, R_CH + (l - 1) * kWidth, 0,
-                                  sW + PL.chb[l - 1], nullptr, 0, true, R_CH + l * kWidth);
-    // the canonical output o into the rows of its delta, read back by each sample's thread
-    warp_fwd<4, kWidth, 0>(sW + PL.cl, 4, wcol, stride, R_CH + (H - 1) * kWidth, 0, sW + PL.clb, nullptr, 0, false,
-                           D_CL);
+      if (active) s = __ldcs(T.samp + j);
+      field_forward<true>(P, T, L, sW, tile, img, s, active, f, F);
     }
     if constexpr (FUSED) {
-      // each slot's (r, g, b, alpha) as train_fwd_kernel forms it, the rays composited in shared
-      // memory by the first warp, and each slot's adjoint back
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (active) {
-        const float o0 = col[D_CL * stride], o1 = col[(D_CL + 1) * stride], o2 = col[(D_CL + 2) * stride],
-                    o3 = col[(D_CL + 3) * stride];
-        const float a = inside ? -expm1f(-softplusf_(o3) * s.w) * fminf(S, 1.f) : 0.f;
-        v = make_float4(sigmoidf_(o0), sigmoidf_(o1), sigmoidf_(o2), a);
-      }
-      if (threadIdx.x < SB) sOut[threadIdx.x] = v;
+      // each slot's (r, g, b, alpha), the rays composited by the first warp, its adjoint back
+      if (threadIdx.x < SB)
+        *reinterpret_cast<float4 *>(tiles + slot_at(threadIdx.x)) =
+            active ? slot_colour(F, s.w) : make_float4(0.f, 0.f, 0.f, 0.f);
       __syncthreads();
-      if (warp == 0) composite_rays(T, sOut, sT, it * RB, RB);
+      if (warp == 0) composite_rays(T, tiles, it * RB, RB);
       __syncthreads();
-      if (active) g4 = sOut[threadIdx.x];
-      if (__ballot_sync(0xffffffffu, active && inside) == 0u) continue;   // no live slot in the warp
+      if (active) g4 = *reinterpret_cast<const float4 *>(tiles + slot_at(threadIdx.x));
+      // no live slot in the warp: its tile is left as it is until the next group's forward
+      if (__ballot_sync(0xffffffffu, active && F.inside) == 0u) continue;
     }
-    active = active && inside;
+    active = active && F.inside;
+    float dcl[4] = {0.f, 0.f, 0.f, 0.f}, dS_alpha = 0.f;
     if (active) {
       // ---------------- alpha, rgb, sigma
-      float *dcl = col + (D_CL) * stride;
-      const float o[4] = {dcl[0], dcl[stride], dcl[2 * stride], dcl[3 * stride]};
-      const float sig = softplusf_(o[3]);
+      const float sig = softplusf_(F.o[3]);
       const float e = expf(-sig * s.w);
-      const float lk = fminf(S, 1.f);
+      const float lk = fminf(F.S, 1.f);
       const float dsig = g4.w * s.w * e * lk;
-      dS_alpha = S < 1.f ? g4.w * -expm1f(-sig * s.w) : 0.f;
+      dS_alpha = F.S < 1.f ? g4.w * -expm1f(-sig * s.w) : 0.f;
       const float gc[3] = {g4.x, g4.y, g4.z};
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const float c = sigmoidf_(o[k]);
-        dcl[k * stride] = gc[k] * c * (1.f - c);
+        const float c = sigmoidf_(F.o[k]);
+        dcl[k] = gc[k] * c * (1.f - c);
       }
-      dcl[3 * stride] = dsig * sigmoidf_(o[3]);
+      dcl[3] = dsig * sigmoidf_(F.o[3]);
     }
-    if (!active)
-      for (int k = 0; k < 4; ++k) col[(D_CL + k) * stride] = 0.f;
+    __syncwarp();   // every lane has its adjoint
+#pragma unroll
+    for (int k = 0; k < 8; ++k) tile[frag_at(k, lane)] = k < 4 ? dcl[k] : 0.f;
     __syncwarp();
-    // ---------------- canonical MLP backward: the warp's 32 samples on the tensor cores, each
-    // layer's weight gradient summed as soon as its delta exists (two delta buffers in turn)
+    float c[2][8][4];
+    auto sign_of = [&](int l) { return reinterpret_cast<const uint2 *>(img + (R.sign + 2 * l) * kTileRow)[lane]; };
+    // ---------------- canonical MLP backward: each layer's weight gradient summed as soon as its
+    // delta is in the tile, then the delta of the layer below
     {
-      int cur = D_B, nxt = D_B + kWidth;
-      warp_back<4, kWidth>(sW + PL.cl, 4, wcol, stride, D_CL, R_CH + (H - 1) * kWidth, cur, false);
-      wgrad4(wcol, stride, R_CH + (H - 1) * kWidth, D_CL, 4, acc, Ly.cl, Ly.clb);
-      for (int l = H - 1; l >= 1; --l) {
-        warp_back<kWidth, kWidth>(sW + PL.ch[l - 1], kPadRow, wcol, stride, cur, R_CH + (l - 1) * kWidth, nxt, false);
-        wgrad64(wcol, stride, R_CH + (l - 1) * kWidth, kWidth, cur, acc, Ly.ch[l - 1], Ly.chb[l - 1], true);
-        const int tmp = cur;
-        cur = nxt;
-        nxt = tmp;
+      wgrad4(tile, img + (R.ch + (H - 1) * kWidth) * kTileRow, 4, acc + Ly.cl, acc + Ly.clb);
+#pragma unroll 1
+      for (int l = H; l >= 1; --l) {   // the delta of layer l is in the tile (l = H: the outputs)
+        const uint2 sg = sign_of(4 + l - 1);
+        if (l < H) wgrad64(L, tile, img + (R.ch + (l - 1) * kWidth) * kTileRow, 8, acc + Ly.ch[l - 1], acc + Ly.chb[l - 1], nullptr);
+        frag_zero(c);
+        frag_back<8>(L, tile, l == H ? 1 : 8, sW + (l == H ? W.cl : W.ch[l - 1]), 8, 0, c);
+        delta_done(L, sg, c, tile);
       }
-      warp_back<kWidth, kMlpIn>(sW + PL.c0, kPadRow, wcol, stride, cur, -1, R_DENC, false);
-      wgrad64(wcol, stride, R_ENC, kMlpIn, cur, acc, Ly.c0, Ly.c0b, true);
+      const int eb = (2 * P.L + 7) >> 3;
+      wgrad64(L, tile, img + R.enc * kTileRow, eb, acc + Ly.c0, acc + Ly.c0b, nullptr);
+      float d[2][4][4];
+      frag_zero(d);
+      frag_back<4>(L, tile, 8, sW + W.c0, kMlpIn / 8, 0, d);
+      frag_store<4>(L, d, tile);
     }
-    __syncwarp();
     float dx0 = 0.f, dx1 = 0.f, dx2 = 0.f;
     {
       // ---------------- hash backward: warp-aggregated scatter-add and dL/dx_final
-      const float p0 = active ? (xf0 - P.bmin[0]) * P.inv_box[0] : 0.f;
-      const float p1 = active ? (xf1 - P.bmin[1]) * P.inv_box[1] : 0.f;
-      const float p2 = active ? (xf2 - P.bmin[2]) * P.inv_box[2] : 0.f;
+      const float p0 = active ? (F.xf0 - P.bmin[0]) * P.inv_box[0] : 0.f;
+      const float p1 = active ? (F.xf1 - P.bmin[1]) * P.inv_box[1] : 0.f;
+      const float p2 = active ? (F.xf2 - P.bmin[2]) * P.inv_box[2] : 0.f;
       for (int l = 0; l < P.L; ++l) {
-        const float da = active ? col[(R_DENC + 2 * l) * stride] : 0.f;
-        const float db = active ? col[(R_DENC + 2 * l + 1) * stride] : 0.f;
+        const float da = active ? tile[frag_at(2 * l, lane)] : 0.f;
+        const float db = active ? tile[frag_at(2 * l + 1, lane)] : 0.f;
         const uint32_t N = P.level_res[l];
         const float fn = (float)N;
         const float q0 = p0 * fn, q1 = p1 * fn, q2 = p2 * fn;
@@ -795,34 +762,44 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P
     float ds0 = dx0, ds1 = dx1, ds2 = dx2;
     if (P.res_enabled) {
       // ---------------- residual MLP backward (x_final = x_skel + x_res), tensor cores
-      float *dr5 = col + D_R5 * stride;
-      dr5[0] = dx0;
-      dr5[stride] = dx1;
-      dr5[2 * stride] = dx2;
-      dr5[3 * stride] = 0.f;
+      const uint32_t fl = qv ? T.frame_id[r] : 0u;   // the frames of the warp's slots: one, if they agree
+      const uint32_t fl0 = __shfl_sync(0xffffffffu, fl, 0);
+      const bool one = __all_sync(0xffffffffu, !qv || fl == fl0) && (q0 < n && (!FUSED || warp * 32u < SB));
       __syncwarp();
-      const int b0 = D_B, b1 = D_B + kWidth;   // delta4 -> b0, delta3 -> b1, delta2 -> b0, delta1 -> b1
-      warp_back<4, kWidth>(sW + PL.r5, 4, wcol, stride, D_R5, R_RH + 3 * kWidth, b0, false);
-      wgrad4(wcol, stride, R_RH + 3 * kWidth, D_R5, 3, acc, Ly.r5, Ly.r5b);
-      warp_back<kWidth, kWidth>(sW + PL.r4, kPadRow, wcol, stride, b0, R_RH + 2 * kWidth, b1, false);
-      warp_back<kWidth, kResGammaPad>(sW + PL.r4 + kWidth * kPadRow, kPadRow, wcol, stride, b0, -1, R_DGAM, false);
-      wgrad64(wcol, stride, R_RH + 2 * kWidth, kWidth, b0, acc, Ly.r4, Ly.r4b, true);
-      wgrad64(wcol, stride, R_GAM, kResGammaPad, b0, acc, Ly.r4 + kWidth * kWidth, 0, false);
-      warp_back<kWidth, kWidth>(sW + PL.r3, kPadRow, wcol, stride, b1, R_RH + 1 * kWidth, b0, false);
-      wgrad64(wcol, stride, R_RH + 1 * kWidth, kWidth, b1, acc, Ly.r3, Ly.r3b, true);
-      warp_back<kWidth, kWidth>(sW + PL.r2, kPadRow, wcol, stride, b0, R_RH + 0 * kWidth, b1, false);
-      wgrad64(wcol, stride, R_RH + 0 * kWidth, kWidth, b0, acc, Ly.r2, Ly.r2b, true);
-      // dL/dgamma += W1_gamma^T delta1 (the pose columns of W1 are reduced per frame below)
-      warp_back<kWidth, kResGammaPad>(sW + PL.r1, kPadRow, wcol, stride, b1, -1, R_DGAM, true);
-      wgrad64(wcol, stride, R_GAM, kResGammaPad, b1, acc, Ly.r1, Ly.r1b, true);
-      {  // per-frame sums of delta1 (for W_Omega): lane owns rows lane, lane + 32
-        const float *d0 = wcol + (b1 + lane) * stride, *d1 = wcol + (b1 + lane + 32) * stride;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) tile[frag_at(k, lane)] = k == 0 ? dx0 : k == 1 ? dx1 : k == 2 ? dx2 : 0.f;
+      __syncwarp();
+      wgrad4(tile, img + (R.rh + 3 * kWidth) * kTileRow, 3, acc + Ly.r5, acc + Ly.r5b);
+#pragma unroll 1
+      for (int l = 4; l >= 1; --l) {   // l = 4: the outputs' delta in the tile; below, hidden layer l + 1's
+        const uint2 sg = sign_of(l - 1);
+        const int IB = l == 3 ? 8 + kGamRows / 8 : 8;
+        if (l < 4)
+          wgrad64(L, tile, img + (R.rh + (l - 1) * kWidth) * kTileRow, 8, acc + (l == 3 ? Ly.r4 : l == 2 ? Ly.r3 : Ly.r2),
+                  acc + (l == 3 ? Ly.r4b : l == 2 ? Ly.r3b : Ly.r2b), nullptr);
+        if (l == 3) {   // layer 4's gamma inputs: weight gradient and the first part of dL/dgamma
+          wgrad64(L, tile, img + R.gam * kTileRow, kGamRows / 8, acc + Ly.r4 + kWidth * kWidth, nullptr, nullptr);
+          float d[2][kGamRows / 8][4];
+          frag_zero(d);
+          frag_back<kGamRows / 8>(L, tile, 8, sW + W.r4, IB, 8, d);
+          float4 *o = reinterpret_cast<float4 *>(img + R.dgam * kTileRow) + lane;
+#pragma unroll
+          for (int k = 0; k < 2 * (kGamRows / 8); ++k)
+            o[32 * k] = make_float4(d[k & 1][k >> 1][0], d[k & 1][k >> 1][1], d[k & 1][k >> 1][2], d[k & 1][k >> 1][3]);
+        }
+        frag_zero(c);
+        frag_back<8>(L, tile, l == 4 ? 1 : 8, sW + (l == 4 ? W.r5 : l == 3 ? W.r4 : l == 2 ? W.r3 : W.r2), IB, 0, c);
+        delta_done(L, sg, c, tile);
+      }
+      wgrad64(L, tile, img + R.gam * kTileRow, kGamRows / 8, acc + Ly.r1, acc + Ly.r1b,
+              one ? accF + fl0 * kWidth : nullptr);
+      if (!one) {  // per-frame sums of delta1 (for W_Omega): lane owns rows lane, lane + 32
+        const float *d0 = tile + lane * kTileRow, *d1 = tile + (lane + 32) * kTileRow;
         int cur = -1;
         float s0 = 0.f, s1 = 0.f;
         for (int sI = 0; sI < 32; ++sI) {
-          const uint32_t jj = q0 + sI;
-          if (jj >= n || (FUSED && (uint32_t)(warp * 32 + sI) >= SB)) break;
-          const int fr = (int)T.frame_id[ray_of(T, jj)];
+          if (q0 + sI >= n || (FUSED && (uint32_t)(warp * 32 + sI) >= SB)) break;
+          const int fr = (int)__shfl_sync(0xffffffffu, fl, sI);
           if (fr != cur) {
             if (cur >= 0) {
               atomicAdd(accF + cur * kWidth + lane, s0);
@@ -831,21 +808,36 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P
             cur = fr;
             s0 = s1 = 0.f;
           }
-          s0 += d0[sI];
-          s1 += d1[sI];
+          const int at = frag_at(lane, sI) - lane * kTileRow;
+          s0 += d0[at];
+          s1 += d1[at];
         }
         if (cur >= 0) {
           atomicAdd(accF + cur * kWidth + lane, s0);
           atomicAdd(accF + cur * kWidth + lane + 32, s1);
         }
       }
-      __syncwarp();
+      {  // dL/dgamma = layer 4's part + W1_gamma^T delta1 (the pose columns of W1: per frame, above)
+        float d[2][kGamRows / 8][4];
+        frag_zero(d);
+        frag_back<kGamRows / 8>(L, tile, 8, sW + W.r1, kGamRows / 8, 0, d);
+        const float4 *o = reinterpret_cast<const float4 *>(img + R.dgam * kTileRow) + lane;
+#pragma unroll
+        for (int k = 0; k < 2 * (kGamRows / 8); ++k) {
+          const float4 v = o[32 * k];
+          d[k & 1][k >> 1][0] += v.x;
+          d[k & 1][k >> 1][1] += v.y;
+          d[k & 1][k >> 1][2] += v.z;
+          d[k & 1][k >> 1][3] += v.w;
+        }
+        frag_store<kGamRows / 8>(L, d, tile);
+      }
       if (active) {
           // through gamma: d gamma / d x_skel
-          const float *dg = col + R_DGAM * stride;
-          const float xh[3] = {(xs0 - P.box_c[0]) * P.box_ih[0], (xs1 - P.box_c[1]) * P.box_ih[1],
-                               (xs2 - P.box_c[2]) * P.box_ih[2]};
-          float dh[3] = {dg[0], dg[stride], dg[2 * stride]};
+          auto dg = [&](int k) { return tile[frag_at(k, lane)]; };
+          const float xh[3] = {(F.xs0 - P.box_c[0]) * P.box_ih[0], (F.xs1 - P.box_c[1]) * P.box_ih[1],
+                               (F.xs2 - P.box_c[2]) * P.box_ih[2]};
+          float dh[3] = {dg(0), dg(1), dg(2)};
           for (int k = 0; k < P.res_freqs; ++k) {
             const float sc = (float)(1 << k);
             const float wk = P.hann[k] * sc * 3.14159265358979f;
@@ -853,7 +845,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P
             for (int a = 0; a < 3; ++a) {
               float sn, cs;
               sincospif(sc * xh[a], &sn, &cs);
-              dh[a] += wk * (dg[(3 + 6 * k + a) * stride] * cs - dg[(6 + 6 * k + a) * stride] * sn);
+              dh[a] += wk * (dg(3 + 6 * k + a) * cs - dg(6 + 6 * k + a) * sn);
             }
           }
           ds0 += dh[0] * P.box_ih[0];
@@ -861,30 +853,32 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P
           ds2 += dh[2] * P.box_ih[2];
       }
     }
+    float *dp = img + R.dp * kTileRow, *xs = img + R.xs * kTileRow;
     {
       // ---------------- inverse-LBS backward: warp-aggregated scatter into the weight volume
       // and, for the pose refiner, dL/dp_i of each candidate p_i = G_i x:
       //   x_skel = sum_i w_i p_i / D,  w_i = W_i(p_i)
       //   dL/dp_i = (w_i / D) dL/dx_skel + dL/dw_i grad W_i(p_i)
-      const float D = fmaxf(S, kEpsW);
+      const float D = fmaxf(F.S, kEpsW);
       // one division per sample: a per-bone quotient with a vanishing numerator (far from the
       // body S, and with it the gradient reaching x_skel, goes to zero) takes the division's
       // slow path 24 times a sample
       const float inv_D = 1.f / D;
-      const float m = S > kEpsW ? 1.f : 0.f;
+      const float m = F.S > kEpsW ? 1.f : 0.f;
+      const float *G = T.fG + (size_t)f * kBones * 12;
       const int R = P.wres, R3 = R * R * R;
       const size_t QC = quad_channel(R);
       if (T.dG && active) {
-        col[(R_XS + 0) * stride] = s.x;
-        col[(R_XS + 1) * stride] = s.y;
-        col[(R_XS + 2) * stride] = s.z;
+        xs[lane] = s.x;
+        xs[kTileRow + lane] = s.y;
+        xs[2 * kTileRow + lane] = s.z;
       }
       for (int i = 0; i < kBones; ++i) {
         const float *g = G + 12 * i;
         const float p0 = fmaf(g[0], s.x, fmaf(g[1], s.y, fmaf(g[2], s.z, g[3])));
         const float p1 = fmaf(g[4], s.x, fmaf(g[5], s.y, fmaf(g[6], s.z, g[7])));
         const float p2 = fmaf(g[8], s.x, fmaf(g[9], s.y, fmaf(g[10], s.z, g[11])));
-        const float dw = (ds0 * (p0 - m * xs0) + ds1 * (p1 - m * xs1) + ds2 * (p2 - m * xs2)) * inv_D + dS_alpha;
+        const float dw = (ds0 * (p0 - m * F.xs0) + ds1 * (p1 - m * F.xs1) + ds2 * (p2 - m * F.xs2)) * inv_D + dS_alpha;
         const float ux = (p0 - P.bmin[0]) * P.vol_scale[0];
         const float uy = (p1 - P.bmin[1]) * P.vol_scale[1];
         const float uz = (p2 - P.bmin[2]) * P.vol_scale[2];
@@ -892,9 +886,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P
           float gx, gy, gz;
           const float w = trilinear_quad_grad(P.wquad + (size_t)i * QC, R, ux, uy, uz, gx, gy, gz);
           const float a = w * inv_D;
-          col[(R_DP + 3 * i + 0) * stride] = fmaf(a, ds0, dw * gx * P.vol_scale[0]);
-          col[(R_DP + 3 * i + 1) * stride] = fmaf(a, ds1, dw * gy * P.vol_scale[1]);
-          col[(R_DP + 3 * i + 2) * stride] = fmaf(a, ds2, dw * gz * P.vol_scale[2]);
+          dp[(3 * i + 0) * kTileRow + lane] = fmaf(a, ds0, dw * gx * P.vol_scale[0]);
+          dp[(3 * i + 1) * kTileRow + lane] = fmaf(a, ds1, dw * gy * P.vol_scale[1]);
+          dp[(3 * i + 2) * kTileRow + lane] = fmaf(a, ds2, dw * gz * P.vol_scale[2]);
         }
         const float fx0 = floorf(ux), fy0 = floorf(uy), fz0 = floorf(uz);
         const bool in_range = fx0 >= -1.f && fy0 >= -1.f && fz0 >= -1.f && fx0 < (float)R && fy0 < (float)R &&
@@ -919,7 +913,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P
       }
     }
     if (T.dG && !active)   // the refiner's reduction reads these rows of every lane
-      for (int q = 0; q < 3 * kBones + 3; ++q) col[(R_DP + q) * stride] = 0.f;
+      for (int q = 0; q < 3 * kBones + 3; ++q) dp[q * kTileRow + lane] = 0.f;   // (xs follows dp)
     __syncwarp();
     if (T.dG) {
       // dL/dG_i of each frame: dR_i += dp_i x^T, dt_i += dp_i over the warp's 32 samples;
@@ -936,8 +930,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
           const int s0 = 8 * ks + t;
-          const float v0 = g < 3 ? wcol[(R_XS + g) * stride + s0] : (g == 3 ? 1.f : 0.f);
-          const float v1 = g < 3 ? wcol[(R_XS + g) * stride + s0 + 4] : (g == 3 ? 1.f : 0.f);
+          const float v0 = g < 3 ? xs[g * kTileRow + s0] : (g == 3 ? 1.f : 0.f);
+          const float v1 = g < 3 ? xs[g * kTileRow + s0 + 4] : (g == 3 ? 1.f : 0.f);
           tf32_split(v0, bh[ks][0], bl[ks][0]);
           tf32_split(v1, bh[ks][1], bl[ks][1]);
         }
@@ -949,10 +943,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P
           for (int ks = 0; ks < 4; ++ks) {
             const int s0 = 8 * ks + t;
             uint32_t ah[4], al[4];
-            tf32_split(o0 < 3 * kBones ? wcol[(R_DP + o0) * stride + s0] : 0.f, ah[0], al[0]);
-            tf32_split(o8 < 3 * kBones ? wcol[(R_DP + o8) * stride + s0] : 0.f, ah[1], al[1]);
-            tf32_split(o0 < 3 * kBones ? wcol[(R_DP + o0) * stride + s0 + 4] : 0.f, ah[2], al[2]);
-            tf32_split(o8 < 3 * kBones ? wcol[(R_DP + o8) * stride + s0 + 4] : 0.f, ah[3], al[3]);
+            tf32_split(o0 < 3 * kBones ? dp[o0 * kTileRow + s0] : 0.f, ah[0], al[0]);
+            tf32_split(o8 < 3 * kBones ? dp[o8 * kTileRow + s0] : 0.f, ah[1], al[1]);
+            tf32_split(o0 < 3 * kBones ? dp[o0 * kTileRow + s0 + 4] : 0.f, ah[2], al[2]);
+            tf32_split(o8 < 3 * kBones ? dp[o8 * kTileRow + s0 + 4] : 0.f, ah[3], al[3]);
             mma_tf32(c, al, bh[ks]);
             mma_tf32(c, ah, bl[ks]);
             mma_tf32(c, ah, bh[ks]);
@@ -967,8 +961,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) train_bwd_kernel(FieldParams P
       } else {
       for (int o = lane; o < kBones * 12; o += 32) {
         const int i = o / 12, rr = (o % 12) >> 2, c = o & 3;
-        const float *dpr = wcol + (R_DP + 3 * i + rr) * stride;
-        const float *xr = wcol + (R_XS + (c < 3 ? c : 0)) * stride;
+        const float *dpr = dp + (3 * i + rr) * kTileRow;
+        const float *xr = xs + (c < 3 ? c : 0) * kTileRow;
         int cur = -1;
         float v = 0.f;
         for (int sI = 0; sI < 32; ++sI) {
@@ -1003,8 +997,8 @@ __global__ void reduce_acc_kernel(const float *__restrict__ wacc, int n_warps, i
   red[e] = s;
 }
 
-// Gradients in the packed master layout (W[out][in], b) from the transposed
-// blob-shaped sums; the joint-angle columns of the residual first layer get
+// Gradients in the packed master layout (W[out][in], b) from the accumulators' sums (fragment
+// order, acc_index); the joint-angle columns of the residual first layer get
 // dL/dW_Omega[j][m] = sum_f (sum of delta1 over frame f)[j] * Omega_f[m].
 struct ScatterArgs {
   MasterOffsets m;
@@ -1022,7 +1016,6 @@ __global__ void scatter_res_kernel(const float *__restrict__ red, const float *_
   const int rout[5] = {kWidth, kWidth, kWidth, kWidth, 3};
   const int wt[5] = {a.b.r1, a.b.r2, a.b.r3, a.b.r4, a.b.r5};
   const int bb[5] = {a.b.r1b, a.b.r2b, a.b.r3b, a.b.r4b, a.b.r5b};
-  const int ostride[5] = {kWidth, kWidth, kWidth, kWidth, 4};
   for (int l = 0; l < 5; ++l) {
     if (e >= a.m.r[l] && e < a.m.rb[l]) {
       const int q = e - a.m.r[l], j = q / rin[l], k = q % rin[l];
@@ -1031,10 +1024,8 @@ __global__ void scatter_res_kernel(const float *__restrict__ red, const float *_
         const int mm = k - a.g;
         v = 0.f;
         for (int f = 0; f < a.n_frames; ++f) v = fmaf(accF[f * kWidth + j], fomega[f * a.pose_dim + mm], v);
-      } else if (l == 3 && k >= kWidth) {
-        v = red[wt[l] + (kWidth + (k - kWidth)) * ostride[l] + j];
       } else {
-        v = red[wt[l] + k * ostride[l] + j];
+        v = red[wt[l] + (l == 4 ? k * 4 + j : acc_index(j, k))];
       }
       g_res[e] = v;
       return;
@@ -1055,10 +1046,9 @@ __global__ void scatter_mlp_kernel(const float *__restrict__ red, ScatterArgs a,
     const int out = l == H ? 4 : kWidth;
     const int wt = l == 0 ? a.b.c0 : (l == H ? a.b.cl : a.b.ch[l - 1]);
     const int bb = l == 0 ? a.b.c0b : (l == H ? a.b.clb : a.b.chb[l - 1]);
-    const int ostride = l == H ? 4 : kWidth;
     if (e >= a.m.c[l] && e < a.m.cb[l]) {
       const int q = e - a.m.c[l], j = q / in, k = q % in;
-      g_mlp[e] = red[wt + k * ostride + j];
+      g_mlp[e] = red[wt + (l == H ? k * 4 + j : acc_index(j, k))];
       return;
     }
     if (e >= a.m.cb[l] && e < a.m.cb[l] + out) {
@@ -1159,8 +1149,20 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
   if ((r = grow(s->t_raycnt, s->tw_rays, (size_t)b->n_rays)) != NR_OK) return r;
   if ((r = grow(s->t_live, s->tw_live, ((size_t)b->n_rays * b->n_samples + 31) / 32)) != NR_OK) return r;
   const Rows rows = make_rows((int)s->hidden);
-  if ((r = grow(s->t_scratch, s->tw_scratch, (size_t)blocks * rows.total * std::max(kFwdThreads, kBwdThreads))) !=
-      NR_OK)
+  const FragLay fl = frag_layout((int)s->hidden);
+  const size_t n_dG = (size_t)s->n_frames * kBones * 12;
+  const bool dG_smem = refine && s->n_frames <= 16;
+  // the warps whose tiles fit beside the weights (sixteen with two hidden layers, eleven with four)
+  const size_t smem_w = sizeof(float) * fl.total, smem_g = dG_smem ? sizeof(float) * n_dG : 0;
+  const size_t tile_b = kTileFloats * sizeof(float);
+  const int warps_f = (int)std::min<size_t>(kTrainThreads / 32, (kTrainSmem - smem_w) / tile_b);
+  const int warps_max = (int)std::min<size_t>(kTrainThreads / 32, (kTrainSmem - smem_w - smem_g) / tile_b);
+  // a step whose rays fit a block whole runs forward, compositing and backward in one kernel
+  // (train_bwd_kernel<true>) over groups of 32 warps / S rays; else the forward and the
+  // compositing adjoint run first
+  const bool fused = !fwd_only && b->n_samples <= (uint32_t)(32 * warps_max);
+  const int warps_b = fused ? (int)((32u * warps_max / b->n_samples * b->n_samples + 31) / 32) : warps_max;
+  if ((r = grow(s->t_scratch, s->tw_scratch, (size_t)blocks * rows.total * kTileRow * (kTrainThreads / 32))) != NR_OK)
     return r;
   const size_t n_acc = (size_t)blocks;                 // one accumulator per block
   if ((r = grow(s->t_wacc, s->tw_acc, n_acc * A)) != NR_OK) return r;
@@ -1178,8 +1180,6 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
   NR_CHECK_CUDA(cudaMemsetAsync(s->g_table, 0, s->n_table * 4, st));
   NR_CHECK_CUDA(cudaMemsetAsync(s->t_wacc, 0, n_acc * A * 4, st));
   NR_CHECK_CUDA(cudaMemsetAsync(s->loss_acc, 0, sizeof(float), st));
-  const size_t n_dG = (size_t)s->n_frames * kBones * 12;
-  const bool dG_smem = refine && s->n_frames <= 16;
   if (refine) {
     if ((r = grow(s->f_dG, s->f_dG_cap, n_dG)) != NR_OK) return r;
     NR_CHECK_CUDA(cudaMemsetAsync(s->f_dG, 0, n_dG * 4, st));
@@ -1216,7 +1216,7 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
   T.rw = rows;
   T.dG = refine ? s->f_dG : nullptr;
   T.dG_smem = dG_smem ? 1 : 0;
-  T.pl = pad_layout(s->lay, (int)s->hidden);
+  T.fl = fl;
   T.pred = b->pred_rgb;
   T.grad_rgb = fwd_only ? nullptr : b->grad_rgb;
   T.forward_only = fwd_only ? 1 : 0;
@@ -1224,13 +1224,10 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
   train_samples_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(T, s->bmin[0], s->bmin[1], s->bmin[2], s->bmax[0],
                                                                      s->bmax[1], s->bmax[2]);
   NR_CHECK_CUDA(cudaGetLastError());
-  const size_t smem_f = sizeof(float) * T.pl.total;
-  // a step whose rays fit a backward block whole runs forward, compositing and backward in one
-  // kernel (train_bwd_kernel<true>); else the forward and the compositing adjoint run first
-  const bool fused = !fwd_only && b->n_samples <= (uint32_t)kBwdThreads;
   if (!fused) {
+    const size_t smem_f = smem_w + warps_f * tile_b;
     NR_CHECK_CUDA(cudaFuncSetAttribute(train_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_f));
-    train_fwd_kernel<<<blocks, kFwdThreads, smem_f, st>>>(P, T);
+    train_fwd_kernel<<<blocks, 32 * warps_f, smem_f, st>>>(P, T);
     NR_CHECK_CUDA(cudaGetLastError());
     train_composite_kernel<<<(b->n_rays + 255) / 256, 256, 0, st>>>(T);
     NR_CHECK_CUDA(cudaGetLastError());
@@ -1244,15 +1241,15 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
     }
     return NR_OK;
   }
-  const size_t smem_b = sizeof(float) * (T.pl.total + (dG_smem ? n_dG : 0)) + (fused ? kBwdThreads * 20 : 0);
+  const size_t smem_b = smem_w + smem_g + warps_b * tile_b;
   if (fused) {
     NR_CHECK_CUDA(
         cudaFuncSetAttribute(train_bwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b));
-    train_bwd_kernel<true><<<blocks, kBwdThreads, smem_b, st>>>(P, T);
+    train_bwd_kernel<true><<<blocks, 32 * warps_b, smem_b, st>>>(P, T);
   } else {
     NR_CHECK_CUDA(
         cudaFuncSetAttribute(train_bwd_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b));
-    train_bwd_kernel<false><<<blocks, kBwdThreads, smem_b, st>>>(P, T);
+    train_bwd_kernel<false><<<blocks, 32 * warps_b, smem_b, st>>>(P, T);
   }
   NR_CHECK_CUDA(cudaGetLastError());
   reduce_acc_kernel<<<(A + 255) / 256, 256, 0, st>>>(s->t_wacc, (int)n_acc, A, s->t_red);
