@@ -240,13 +240,15 @@ struct nr_subject {
   size_t tw_live = 0;                // capacity of t_live
   size_t tw_acc = 0;                 // capacity of t_wacc (floats)
   size_t tw_red = 0, tw_scratch = 0;  // capacities of t_red, t_scratch (floats)
+  size_t tw_gquad = 0;               // capacity of t_gquad
   float4 *t_samp = nullptr;          // [n_rays * S] x, y, z, delta
   float4 *t_out = nullptr;           // [n_rays * S] (r, g, b, alpha), then (dL/dc, dL/dalpha)
   float *t_T = nullptr;              // [n_rays * S] transmittance before each sample
   uint32_t *t_raycnt = nullptr;      // [n_rays] S if the ray meets the box, else 0
   uint32_t *t_live = nullptr;        // [n_rays * S / 32] per 32 thread slots: which carry gradient
-  float *t_scratch = nullptr;        // per-thread activation columns of the backward kernel
-  float *t_wacc = nullptr;           // per-warp private MLP-gradient accumulators
+  float *t_scratch = nullptr;        // per-warp images of the activations that the backward reads
+  float4 *t_gquad = nullptr;         // corner-block sums of the weight-volume gradient
+  float *t_wacc = nullptr;           // per-block MLP-gradient accumulators
   float *t_red = nullptr;            // their sum (float32 blob layout + per-frame bias rows)
   float *loss_acc = nullptr;         // [1]
   float *f_dbias1 = nullptr;         // [F][64] (unused, kept for layout)

@@ -696,7 +696,7 @@ static void free_subject(nr_subject *s) {
                   s->g_res,  s->adam_m,  s->adam_v,   s->table16,  s->dense_quad, s->r_scratch, s->blob,      s->tc_bf16,   s->tc_f16,
                   s->d_G,    s->d_omega, s->d_bias1,  s->ellip,    s->bits,      s->f_G,       s->f_omega,
                   s->f_bias1, s->f_cam,  s->samp,     s->samp_out, s->ray_range, s->counter,   s->out_stage,
-                  s->t_samp, s->t_out,   s->t_T,      s->t_raycnt, s->t_live,   s->t_scratch, s->t_wacc,    s->t_red,
+                  s->t_samp, s->t_out,   s->t_T,      s->t_raycnt, s->t_live,   s->t_scratch, s->t_gquad, s->t_wacc,    s->t_red,
                   s->loss_acc, s->f_dbias1, s->fp8_blob, s->fp8_scales, s->fp8_jobs, s->fp8_G,
                   s->t5_bf16,  s->t5_f16,  s->t5_fp8,  s->t5_err,  s->ray_state, s->ray_next, s->canon_bits, s->occ_raw,
                   s->ref, s->g_ref, s->ref_m, s->ref_v, s->f_root, s->f_dG, s->f_omega_o,

@@ -164,17 +164,24 @@ __device__ __forceinline__ void frag_mma(const FragLane &L, const float *tile, i
       tf32_split(x[L.a[2 * m + 1] + 4 * kTileRow], ah[m][3], al[m][3]);
     }
     const float *w = W + ks * ks_step;
+    // two output tiles at a time: four independent accumulators lie between the dependent MMAs
+    // of one (21 cycles apart at best)
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      uint32_t bh[2], bl[2];
-      tf32_split(w[n * n_step + w0], bh[0], bl[0]);
-      tf32_split(w[n * n_step + w1], bh[1], bl[1]);
+    for (int n = 0; n < NT; n += 2) {
+      uint32_t bh[2][2], bl[2][2];
 #pragma unroll
-      for (int m = 0; m < 2; ++m) mma_tf32(c[m][n], ah[m], bl);
+      for (int e = 0; e < 2; ++e)
+        if (n + e < NT) {
+          tf32_split(w[(n + e) * n_step + w0], bh[e][0], bl[e][0]);
+          tf32_split(w[(n + e) * n_step + w1], bh[e][1], bl[e][1]);
+        }
 #pragma unroll
-      for (int m = 0; m < 2; ++m) mma_tf32(c[m][n], al[m], bh);
+      for (int p = 0; p < 3; ++p)
 #pragma unroll
-      for (int m = 0; m < 2; ++m) mma_tf32(c[m][n], ah[m], bh);
+        for (int e = 0; e < 2; ++e)
+#pragma unroll
+          for (int m = 0; m < 2; ++m)
+            if (n + e < NT) mma_tf32(c[m][n + e], p == 1 ? al[m] : ah[m], p == 0 ? bl[e] : bh[e]);
     }
   }
 }

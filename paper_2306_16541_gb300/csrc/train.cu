@@ -25,6 +25,7 @@
 #include <string.h>
 
 #include "field.cuh"
+#include "gather.cuh"
 #include "render.cuh"
 #include "tf32.cuh"
 
@@ -32,6 +33,7 @@ namespace nr {
 
 constexpr int kTrainThreads = 512;   // at most: sixteen warps of 128 registers
 constexpr size_t kTrainSmem = 227 * 1024;
+constexpr size_t kQuadBytes = 512;
 
 // Rows (of 32 floats) of a warp's global image, sized for the subject's hidden depth H.
 struct Rows {
@@ -78,6 +80,7 @@ struct TrainDev {
   float *loss;
   float2 *g_table;
   float *g_wvol;
+  float4 *g_quad;         // corner-block sums of the weight-volume gradient (layout of wquad), or NULL
   float *scratch, *wacc;
   int acc_floats;         // floats per block accumulator
   int n_frames;
@@ -418,8 +421,16 @@ __device__ __noinline__ void field_forward(const FieldParams &P, const TrainDev 
     if (k < kGamRows) tile[frag_at(k, lane)] = v;
   };
   F.xs0 = F.xs1 = F.xs2 = F.S = 0.f;
+  {  // four bones' corner blocks in flight at a time (the bits of lbs_warp)
+    const float *G = T.fG + (size_t)f * kBones * 12;
+    LbsState st;
+    st.x0 = s.x;
+    st.x1 = s.y;
+    st.x2 = s.z;
+    lbs_begin(P, G, nullptr, st, active);
+    lbs_end(P, G, st, F.xs0, F.xs1, F.xs2, F.S);
+  }
   if (active) {
-    lbs_warp(P, T.fG + (size_t)f * kBones * 12, s.x, s.y, s.z, F.xs0, F.xs1, F.xs2, F.S);
     if (P.res_enabled) pos_enc(P, F.xs0, F.xs1, F.xs2, put);
   } else if (P.res_enabled) {
     for (int q = 0; q < kGamRows; ++q) put(q, 0.f);
@@ -725,6 +736,10 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams
         const float fr[3] = {q0 - a0, q1 - a1, q2 - a2};
         HashCell c;
         hash_cell(P, l, p0, p1, p2, c);
+        float2 tv[8];   // the corners, loaded before the exchange below
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          tv[k] = active ? __ldg(P.table32 + (size_t)l * (P.T_mask + 1) + c.idx[k]) : make_float2(0.f, 0.f);
         float v[16];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -741,8 +756,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams
           float gp0 = 0.f, gp1 = 0.f, gp2 = 0.f;
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
-            const float2 tv = __ldg(P.table32 + (size_t)l * (P.T_mask + 1) + c.idx[k]);
-            const float sv = tv.x * da + tv.y * db;
+            const float sv = tv[k].x * da + tv[k].y * db;
             const float wx = (k & 1) ? fr[0] : 1.f - fr[0], wy = ((k >> 1) & 1) ? fr[1] : 1.f - fr[1],
                         wz = (k >> 2) ? fr[2] : 1.f - fr[2];
             const float sx = (k & 1) ? 1.f : -1.f, sy = ((k >> 1) & 1) ? 1.f : -1.f, sz = (k >> 2) ? 1.f : -1.f;
@@ -902,12 +916,19 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams
           v[c] = dw * (((c & 1) ? fx : 1.f - fx) * (((c >> 1) & 1) ? fy : 1.f - fy) * ((c >> 2) ? fz : 1.f - fz));
         const uint32_t key = (uint32_t)(ix + 1) | ((uint32_t)(iy + 1) << 10) | ((uint32_t)(iz + 1) << 20);
         if (run_sum<8>(key, 0u, valid, v)) {
-          float *chg = T.g_wvol + (size_t)i * R3;
+          if (T.g_quad) {   // the cell's two corner blocks, one 16-byte add each
+            const int R1 = R + 1;
+            float4 *e = T.g_quad + (size_t)i * QC + ((iz + 1) * R1 + (iy + 1)) * R1 + (ix + 1);
+            atomicAdd(e, make_float4(v[0], v[1], v[2], v[3]));
+            atomicAdd(e + R1 * R1, make_float4(v[4], v[5], v[6], v[7]));
+          } else {
+            float *chg = T.g_wvol + (size_t)i * R3;
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            const int ax = ix + (c & 1), ay = iy + ((c >> 1) & 1), az = iz + (c >> 2);
-            if (ax < 0 || ay < 0 || az < 0 || ax >= R || ay >= R || az >= R) continue;
-            atomicAdd(chg + (az * R + ay) * R + ax, v[c]);
+            for (int c = 0; c < 8; ++c) {
+              const int ax = ix + (c & 1), ay = iy + ((c >> 1) & 1), az = iz + (c >> 2);
+              if (ax < 0 || ay < 0 || az < 0 || ax >= R || ay >= R || az >= R) continue;
+              atomicAdd(chg + (az * R + ay) * R + ax, v[c]);
+            }
           }
         }
       }
@@ -985,6 +1006,20 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams
     __syncthreads();
     for (int i = threadIdx.x; i < T.n_frames * kBones * 12; i += blockDim.x)
       if (sdG[i] != 0.f) atomicAdd(T.dG + i, sdG[i]);
+  }
+}
+
+// The weight-volume gradient from its corner-block sums: a vertex lies in up to four blocks of its
+// plane (as corner 0 of its own cell, 1 of the cell before in x, 2 in y, 3 in both).
+__global__ void __launch_bounds__(256) fold_quad_kernel(const float4 *__restrict__ quad, int R, float *__restrict__ g) {
+  const size_t QC = quad_channel(R), R3 = (size_t)R * R * R;
+  const size_t n = R3 * kBones;
+  const int R1 = R + 1;
+  for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+    const int c = (int)(e / R3), v = (int)(e % R3);
+    const int x = v % R, y = (v / R) % R, z = v / (R * R);
+    const float4 *q = quad + (size_t)c * QC + ((size_t)(z + 1) * R1 + y) * R1 + x;
+    g[e] = (__ldg(&q[R1 + 1].x) + __ldg(&q[R1].y)) + (__ldg(&q[1].z) + __ldg(&q[0].w));
   }
 }
 
@@ -1162,6 +1197,11 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
   // compositing adjoint run first
   const bool fused = !fwd_only && b->n_samples <= (uint32_t)(32 * warps_max);
   const int warps_b = fused ? (int)((32u * warps_max / b->n_samples * b->n_samples + 31) / 32) : warps_max;
+  // Corner-block sums of the weight-volume gradient take two 16-byte adds a cell instead of eight
+  // 4-byte ones, for a buffer to clear and fold (4 x 24 / 25 of the volume's bytes and a shell):
+  // taken while that is below kQuadBytes per sample.
+  const size_t n_quad = quad_channel((int)s->wres) * kBones;
+  const bool quad = !fwd_only && n_quad * sizeof(float4) <= kQuadBytes * n;
   if ((r = grow(s->t_scratch, s->tw_scratch, (size_t)blocks * rows.total * kTileRow * (kTrainThreads / 32))) != NR_OK)
     return r;
   const size_t n_acc = (size_t)blocks;                 // one accumulator per block
@@ -1176,7 +1216,14 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
     NR_CHECK_CUDA(cudaMemsetAsync(s->adam_v, 0, s->n_params_total * 4, st));
     s->adam_t = 0;
   }
-  NR_CHECK_CUDA(cudaMemsetAsync(s->g_wvol, 0, s->n_wvol * 4, st));
+  if (quad) {
+    if ((r = grow(s->t_gquad, s->tw_gquad, n_quad)) != NR_OK) return r;
+    NR_CHECK_CUDA(cudaMemsetAsync(s->t_gquad, 0, n_quad * sizeof(float4), st));
+    const size_t bones = (size_t)kBones * s->wres * s->wres * s->wres;   // the channels that the fold writes
+    NR_CHECK_CUDA(cudaMemsetAsync(s->g_wvol + bones, 0, (s->n_wvol - bones) * 4, st));
+  } else {
+    NR_CHECK_CUDA(cudaMemsetAsync(s->g_wvol, 0, s->n_wvol * 4, st));
+  }
   NR_CHECK_CUDA(cudaMemsetAsync(s->g_table, 0, s->n_table * 4, st));
   NR_CHECK_CUDA(cudaMemsetAsync(s->t_wacc, 0, n_acc * A * 4, st));
   NR_CHECK_CUDA(cudaMemsetAsync(s->loss_acc, 0, sizeof(float), st));
@@ -1209,6 +1256,7 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
   T.loss = s->loss_acc;
   T.g_table = reinterpret_cast<float2 *>(s->g_table);
   T.g_wvol = s->g_wvol;
+  T.g_quad = quad ? s->t_gquad : nullptr;
   T.scratch = s->t_scratch;
   T.wacc = s->t_wacc;
   T.acc_floats = A;
@@ -1252,6 +1300,11 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
     train_bwd_kernel<false><<<blocks, 32 * warps_b, smem_b, st>>>(P, T);
   }
   NR_CHECK_CUDA(cudaGetLastError());
+  if (quad) {
+    const int nb = (int)std::min<size_t>(((size_t)kBones * s->wres * s->wres * s->wres + 255) / 256, (size_t)blocks * 8);
+    fold_quad_kernel<<<nb, 256, 0, st>>>(s->t_gquad, (int)s->wres, s->g_wvol);
+    ++launched;
+  }
   reduce_acc_kernel<<<(A + 255) / 256, 256, 0, st>>>(s->t_wacc, (int)n_acc, A, s->t_red);
   ScatterArgs sa{};
   sa.m = master_offsets(s);
