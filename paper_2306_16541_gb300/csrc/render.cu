@@ -12,23 +12,19 @@ namespace nr {
 
 // ------------------------------------------------------------ ray marching
 // One thread per ray.  Pass 1 counts the live samples (midpoint of each of the
-// S bins, kept when its occupancy cell is set); a warp-wide prefix sum and one
-// atomic per warp reserve a contiguous run of the sample queue; pass 2 writes
-// each live sample's position and spacing in ray order.
+// S bins, kept when its occupancy cell is set); one atomic per warp reserves a
+// run of the sample queue for its 32 rays; pass 2 writes each live sample's
+// position and spacing, the warp's rays step by step (StepQueue).
 //   D = (hi - lo) / S,  t_i = lo + ((i + 0.5) D),  x_k = o_k + (t_i d_k)
 //   h_k = (bmax_k - bmin_k) / G,  c_k = clamp(floor((x_k - bmin_k) / h_k), 0, G - 1)
 __global__ void __launch_bounds__(256) march_kernel(CamParams cam, MarchParams mp, float4 *__restrict__ samp,
                                                     uint2 *__restrict__ ray_range, uint32_t *__restrict__ counter) {
   const uint32_t r = mp.ray0 + blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = r < mp.ray_end;
-  const uint32_t lane = threadIdx.x & 31;
   float o[3], d[3], lo = 0.f, hi = 0.f;
   camera_origin(cam, o);
-  bool hit = false;
-  if (valid) {
-    const uint32_t u = r % cam.width, v = r / cam.width;
-    hit = ray_setup(cam, o, mp.bmin, mp.bmax, u, v, d, lo, hi);
-  }
+  uint32_t u, v;
+  const bool hit = valid && ray_pixel(cam, r, u, v) && ray_setup(cam, o, mp.bmin, mp.bmax, u, v, d, lo, hi);
   const uint32_t S = cam.n_samples;
   const float D = __fdiv_rn(__fsub_rn(hi, lo), (float)S);
   const int G = mp.grid;
@@ -56,24 +52,20 @@ __global__ void __launch_bounds__(256) march_kernel(CamParams cam, MarchParams m
       count += live(i, x) ? 1u : 0u;
     }
   }
-  // warp-level exclusive scan of counts, one atomic per warp
-  uint32_t incl = count;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= (uint32_t)off) incl += y;
-  }
-  const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+  const uint32_t total = __reduce_add_sync(0xffffffffu, count), most = __reduce_max_sync(0xffffffffu, count);
   uint32_t base = 0;
-  if (lane == 31) base = atomicAdd(counter, total);
-  base = __shfl_sync(0xffffffffu, base, 31);
-  const uint32_t off = base + incl - count;
-  if (valid) ray_range[r - mp.ray0] = make_uint2(off, count);
-  if (count) {
-    uint32_t w = off;
-    for (uint32_t i = 0; i < S; ++i) {
+  if ((threadIdx.x & 31) == 0 && total) base = atomicAdd(counter, total);
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (valid) ray_range[r - mp.ray0] = make_uint2(base, count);
+  StepQueue Q(base);
+  uint32_t e = 0;
+  for (uint32_t i = 0; i < most; ++i) {
+    const uint32_t w = Q.place(i < count);
+    if (i < count) {
       float x[3];
-      if (live(i, x)) samp[w++] = make_float4(x[0], x[1], x[2], D);
+      while (!live(e, x)) ++e;
+      ++e;
+      samp[w] = make_float4(x[0], x[1], x[2], D);
     }
   }
 }
@@ -237,24 +229,47 @@ nr_status launch_occupancy_field(const FieldParams &P, int mode, uint32_t *bits,
 // --------------------------------------------------------------- composite
 // Eq. 3 front to back: T_0 = 1, w_i = T_i alpha_i, C += w_i c_i,
 // T_{i+1} = T_i (1 - alpha_i); stop once T < t_min (early ray termination,
-// Sec. 2.3).  Pixel = (C + T bg, 1 - T).  One thread per ray.
-__global__ void __launch_bounds__(256) composite_kernel(const uint2 *__restrict__ ray_range,
+// Sec. 2.3).  Pixel = (C + T bg, 1 - T).  One thread per ray; the warp walks the queue's steps
+// (StepQueue), so its loads are of neighbouring samples, four steps' loads ahead of the sums.
+struct RayFold {
+  float c0, c1, c2, T;
+  bool done;
+};
+__device__ __forceinline__ void fold_steps(const float4 *__restrict__ so, uint2 rr, float t_min, RayFold &F) {
+  const uint32_t most = __reduce_max_sync(0xffffffffu, rr.y);
+  StepQueue Q(__shfl_sync(0xffffffffu, rr.x, 0));
+  for (uint32_t i = 0; i < most; i += 4) {
+    float4 v[4];
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k) {
+      const bool has = i + k < rr.y;
+      const uint32_t p = Q.place(has);
+      if (has && !F.done) v[k] = so[p];
+    }
+#pragma unroll
+    for (uint32_t k = 0; k < 4; ++k)
+      if (i + k < rr.y && !F.done) {
+        const float w = F.T * v[k].w;
+        F.c0 = fmaf(w, v[k].x, F.c0);
+        F.c1 = fmaf(w, v[k].y, F.c1);
+        F.c2 = fmaf(w, v[k].z, F.c2);
+        F.T *= 1.f - v[k].w;
+        F.done = F.T < t_min;
+      }
+    if (__all_sync(0xffffffffu, F.done || i + 4 >= rr.y)) break;
+  }
+}
+
+__global__ void __launch_bounds__(256) composite_kernel(CamParams cam, uint32_t ray0,
+                                                        const uint2 *__restrict__ ray_range,
                                                         const float4 *__restrict__ so, uint32_t n_rays, float t_min,
                                                         float bg0, float bg1, float bg2, float4 *__restrict__ out) {
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n_rays) return;
-  const uint2 rr = ray_range[r];
-  float T = 1.f, c0 = 0.f, c1 = 0.f, c2 = 0.f;
-  for (uint32_t i = 0; i < rr.y; ++i) {
-    const float4 v = so[rr.x + i];
-    const float w = T * v.w;
-    c0 = fmaf(w, v.x, c0);
-    c1 = fmaf(w, v.y, c1);
-    c2 = fmaf(w, v.z, c2);
-    T *= 1.f - v.w;
-    if (T < t_min) break;
-  }
-  out[r] = make_float4(fmaf(T, bg0, c0), fmaf(T, bg1, c1), fmaf(T, bg2, c2), 1.f - T);
+  RayFold F{0.f, 0.f, 0.f, 1.f, false};
+  fold_steps(so, r < n_rays ? ray_range[r] : make_uint2(0u, 0u), t_min, F);
+  uint32_t u, v;
+  if (r < n_rays && ray_pixel(cam, ray0 + r, u, v))
+    out[(size_t)v * cam.width + u] = make_float4(fmaf(F.T, bg0, F.c0), fmaf(F.T, bg1, F.c1), fmaf(F.T, bg2, F.c2), 1.f - F.T);
 }
 
 // ------------------------------------------------------- round-based ERT
@@ -287,15 +302,12 @@ __global__ void __launch_bounds__(256) march_round_kernel(CamParams cam, MarchPa
                                                           uint32_t *__restrict__ next) {
   const uint32_t r = mp.ray0 + blockIdx.x * blockDim.x + threadIdx.x;
   const bool valid = r < mp.ray_end;
-  const uint32_t lane = threadIdx.x & 31;
   float o[3], d[3], lo = 0.f, hi = 0.f;
   camera_origin(cam, o);
   const uint32_t st0 = valid ? next[r - mp.ray0] : kRayDone;
-  bool active = !(st0 & kRayDone);
-  if (active) {
-    const uint32_t u = r % cam.width, v = r / cam.width;
-    active = ray_setup(cam, o, mp.bmin, mp.bmax, u, v, d, lo, hi);
-  }
+  uint32_t u, v;
+  const bool active = !(st0 & kRayDone) && ray_pixel(cam, r, u, v) &&
+                      ray_setup(cam, o, mp.bmin, mp.bmax, u, v, d, lo, hi);
   const uint32_t S = cam.n_samples;
   const float D = __fdiv_rn(__fsub_rn(hi, lo), (float)S);
   const int G = mp.grid;
@@ -334,43 +346,34 @@ __global__ void __launch_bounds__(256) march_round_kernel(CamParams cam, MarchPa
     }
     i_end = i;
   }
-  uint32_t incl = count;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= (uint32_t)off) incl += y;
-  }
-  const uint32_t wtotal = __shfl_sync(0xffffffffu, incl, 31);
+  const uint32_t wtotal = __reduce_add_sync(0xffffffffu, count), most = __reduce_max_sync(0xffffffffu, count);
   uint32_t base = 0;
-  if (lane == 31 && wtotal) {
+  if ((threadIdx.x & 31) == 0 && wtotal) {
     base = atomicAdd(counter, wtotal);
     if (total) atomicAdd(total, wtotal);
   }
-  base = __shfl_sync(0xffffffffu, base, 31);
-  const uint32_t off = base + incl - count;
+  base = __shfl_sync(0xffffffffu, base, 0);
   if (valid) {
-    ray_range[r - mp.ray0] = make_uint2(off, count);
+    ray_range[r - mp.ray0] = make_uint2(base, count);
     if (!(st0 & kRayDone)) next[r - mp.ray0] = i_end;
   }
-  if (count) {
-    uint32_t w = off;
-    if (i_end - i0 <= 128u) {   // the flags hold every slot tested: only positions are recomputed
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        uint64_t bits = q ? m1 : m0;
-        while (bits) {
-          const uint32_t e = 64u * q + (uint32_t)(__ffsll((long long)bits) - 1);
-          bits &= bits - 1u;
-          float x[3];
-          pos(i0 + e, x);
-          samp[w++] = make_float4(x[0], x[1], x[2], D);
-        }
+  StepQueue Q(base);
+  const bool flags = i_end - i0 <= 128u;   // they hold every slot tested: only positions are recomputed
+  uint32_t e = i0;
+  for (uint32_t i = 0; i < most; ++i) {
+    const uint32_t w = Q.place(i < count);
+    if (i < count) {
+      float x[3];
+      if (flags) {
+        const bool low = m0 != 0u;
+        uint64_t &m = low ? m0 : m1;
+        pos(i0 + (low ? 0u : 64u) + (uint32_t)(__ffsll((long long)m) - 1), x);
+        m &= m - 1u;
+      } else {
+        while (!live(e, x)) ++e;
+        ++e;
       }
-    } else {
-      for (uint32_t i = i0; w < off + count; ++i) {
-        float x[3];
-        if (live(i, x)) samp[w++] = make_float4(x[0], x[1], x[2], D);
-      }
+      samp[w] = make_float4(x[0], x[1], x[2], D);
     }
   }
 }
@@ -382,36 +385,29 @@ __global__ void __launch_bounds__(256) composite_round_kernel(const uint2 *__res
                                                               uint32_t *__restrict__ next, uint32_t *__restrict__ counter) {
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r == 0) *counter = 0u;   // the round's field launch has read it: cleared for the next march
-  if (r >= n_rays) return;
-  const uint32_t nx = next[r];
-  if (nx & kRayDone) return;
-  float4 c = state[r];
-  bool done = false;
-  const uint2 rr = ray_range[r];
-  for (uint32_t i = 0; i < rr.y; ++i) {
-    const float4 v = so[rr.x + i];
-    const float w = c.w * v.w;
-    c.x = fmaf(w, v.x, c.x);
-    c.y = fmaf(w, v.y, c.y);
-    c.z = fmaf(w, v.z, c.z);
-    c.w *= 1.f - v.w;
-    if (c.w < t_min) {
-      done = true;
-      break;
-    }
+  const uint32_t nx = r < n_rays ? next[r] : kRayDone;
+  const bool open = !(nx & kRayDone);
+  RayFold F{0.f, 0.f, 0.f, 1.f, false};
+  uint2 rr = r < n_rays ? ray_range[r] : make_uint2(0u, 0u);   // a retired ray's count is 0
+  if (open) {
+    const float4 c = state[r];
+    F = RayFold{c.x, c.y, c.z, c.w, false};
   }
-  state[r] = c;
-  if (done || nx >= S) next[r] = nx | kRayDone;
+  fold_steps(so, rr, t_min, F);
+  if (!open) return;
+  state[r] = make_float4(F.c0, F.c1, F.c2, F.T);
+  if (F.done || nx >= S) next[r] = nx | kRayDone;
 }
 
 __global__ void add_u32_kernel(uint32_t *__restrict__ acc, const uint32_t *__restrict__ v) { *acc += *v; }
 
-__global__ void finalize_rays_kernel(const float4 *__restrict__ state, uint32_t n_rays, float bg0, float bg1, float bg2,
-                                     float4 *__restrict__ out) {
+__global__ void finalize_rays_kernel(CamParams cam, uint32_t ray0, const float4 *__restrict__ state, uint32_t n_rays,
+                                     float bg0, float bg1, float bg2, float4 *__restrict__ out) {
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n_rays) return;
+  uint32_t u, v;
+  if (r >= n_rays || !ray_pixel(cam, ray0 + r, u, v)) return;
   const float4 c = state[r];
-  out[r] = make_float4(fmaf(c.w, bg0, c.x), fmaf(c.w, bg1, c.y), fmaf(c.w, bg2, c.z), 1.f - c.w);
+  out[(size_t)v * cam.width + u] = make_float4(fmaf(c.w, bg0, c.x), fmaf(c.w, bg1, c.y), fmaf(c.w, bg2, c.z), 1.f - c.w);
 }
 
 int num_sms(int device) {
@@ -500,7 +496,11 @@ static nr_status check_opts(const nr_render_opts *o) {
   return NR_OK;
 }
 
-CamParams cam_params(const nr_camera *c) {
+uint32_t ray_slots(const CamParams &c) {
+  return c.patch_cols ? c.patch_cols * ((c.height + 3) / 4) * 32 : c.width * c.height;
+}
+
+CamParams cam_params(const nr_camera *c, uint64_t max_slots) {
   CamParams p{};
   memcpy(p.R, c->R, sizeof(p.R));
   memcpy(p.t, c->t, sizeof(p.t));
@@ -513,6 +513,9 @@ CamParams cam_params(const nr_camera *c) {
   p.width = c->width;
   p.height = c->height;
   p.n_samples = c->n_samples;
+  const uint64_t n = (uint64_t)c->width * c->height, cols = (c->width + 7) / 8;
+  const uint64_t slots = cols * ((c->height + 3) / 4) * 32;
+  p.patch_cols = slots <= std::min<uint64_t>(max_slots, n + n / 8) ? (uint32_t)cols : 0u;
   return p;
 }
 
@@ -551,13 +554,14 @@ uint32_t round_samples(const nr_camera *cam, const nr_render_opts *opts) {
 nr_status render_rays(const nr_subject *s, const FieldParams &P, const uint32_t *bits, const nr_camera *cam,
                       const nr_render_opts *opts, const FrameWork &w, float4 *dst, cudaStream_t st, int mma_path,
                       Prof *prof) {
-  const CamParams C = cam_params(cam);
-  const uint32_t n_rays = cam->width * cam->height;
+  const CamParams C = cam_params(cam, UINT64_MAX);   // any number of rays: they are taken in chunks
+  const uint32_t n_rays = ray_slots(C);
   const uint32_t S = cam->n_samples;
   const uint32_t k = round_samples(cam, opts);
   const bool rounds = k < S || opts->t_min > 0.f;
-  const uint32_t chunk = (uint32_t)std::min<uint64_t>(std::min<uint64_t>(n_rays, w.cap_rays),
-                                                      std::max<uint64_t>(1, w.cap_samples / k));
+  uint32_t chunk = (uint32_t)std::min<uint64_t>(std::min<uint64_t>(n_rays, w.cap_rays),
+                                                std::max<uint64_t>(1, w.cap_samples / k));
+  if (chunk > 32 && chunk < n_rays) chunk &= ~31u;     // whole patches
   if (chunk == 0 || (rounds && (!w.state || !w.next))) {
     set_error("render: workspace too small");
     return NR_EINVAL;
@@ -612,14 +616,14 @@ nr_status render_rays(const nr_subject *s, const FieldParams &P, const uint32_t 
         composite_round_kernel<<<nb, 256, 0, st>>>(w.ray_range, w.samp_out, nr_, opts->t_min, S, w.state, w.next,
                                                    w.counter);
       else
-        composite_kernel<<<nb, 256, 0, st>>>(w.ray_range, w.samp_out, nr_, opts->t_min, cam->bg[0], cam->bg[1],
-                                             cam->bg[2], dst + r0);
+        composite_kernel<<<nb, 256, 0, st>>>(C, r0, w.ray_range, w.samp_out, nr_, opts->t_min, cam->bg[0], cam->bg[1],
+                                             cam->bg[2], dst);
       NR_CHECK_CUDA(cudaGetLastError());
       NR_CHECK_CUDA(mark(2));
       count_launches(3);
     }
     if (rounds) {
-      finalize_rays_kernel<<<nb, 256, 0, st>>>(w.state, nr_, cam->bg[0], cam->bg[1], cam->bg[2], dst + r0);
+      finalize_rays_kernel<<<nb, 256, 0, st>>>(C, r0, w.state, nr_, cam->bg[0], cam->bg[1], cam->bg[2], dst);
       NR_CHECK_CUDA(cudaGetLastError());
       count_launches(1);
     }
@@ -671,7 +675,8 @@ extern "C" nr_status nr_render(nr_subject *s, const nr_camera *cam, const nr_ren
   // chunk the rays so that the worst-case sample queue of a round stays below 2^26 entries
   const uint64_t max_samples = 1ull << 26;
   const uint32_t k = round_samples(cam, opts);
-  const uint32_t chunk = (uint32_t)std::min<uint64_t>(n_rays, std::max<uint64_t>(256, max_samples / k));
+  const uint32_t chunk = (uint32_t)std::min<uint64_t>(ray_slots(cam_params(cam, UINT64_MAX)),
+                                                      std::max<uint64_t>(256, max_samples / k));
   if ((r = grow_workspace(s, chunk, (size_t)chunk * k)) != NR_OK) return r;
   cudaPointerAttributes attr{};
   const bool dev_out = cudaPointerGetAttributes(&attr, out_rgba) == cudaSuccess && attr.type == cudaMemoryTypeDevice;

@@ -18,6 +18,37 @@ struct CamParams {
   float R[9], t[3];
   float fx, fy, cx, cy, t_near, t_far;
   uint32_t width, height, n_samples;
+  uint32_t patch_cols;           // rays in patches of 8 x 4 pixels: patches per row; 0: in row order
+};
+
+// Rays are numbered in patches of 8 x 4 pixels where the image allows it, so that a warp's 32 rays
+// are neighbours both ways: at one depth their samples then lie in one or a few cells of the weight
+// volume and of the coarser hash levels.  r's pixel; false for a number past the image's edge.
+__device__ __forceinline__ bool ray_pixel(const CamParams &c, uint32_t r, uint32_t &u, uint32_t &v) {
+  if (!c.patch_cols) {
+    u = r % c.width;
+    v = r / c.width;
+    return true;
+  }
+  const uint32_t p = r >> 5;
+  u = (p % c.patch_cols) * 8 + (r & 7);
+  v = (p / c.patch_cols) * 4 + ((r >> 3) & 3);
+  return u < c.width && v < c.height;
+}
+
+// The samples of a warp's 32 rays lie in the queue step by step: the first samples of all rays
+// that have one, then the second ones, and so on, from `base`; neighbouring lanes of the field
+// kernel thus hold neighbouring rays' samples at one depth instead of one ray's samples in depth.
+// Walks the steps in order: place(i, has) is the queue place of this lane's sample i (a ray with
+// `count` samples has samples 0 .. count - 1).  Every lane of the warp must take part.
+struct StepQueue {
+  uint32_t at, below;
+  __device__ __forceinline__ StepQueue(uint32_t base) : at(base), below((1u << (threadIdx.x & 31)) - 1u) {}
+  __device__ __forceinline__ uint32_t place(bool has) {
+    const uint32_t m = __ballot_sync(0xffffffffu, has), p = at + __popc(m & below);
+    at += __popc(m);
+    return p;
+  }
 };
 
 struct MarchParams {
@@ -81,8 +112,9 @@ __device__ __forceinline__ bool ray_setup(const CamParams &c, const float o[3], 
 
 __global__ void march_kernel(CamParams cam, MarchParams mp, float4 *__restrict__ samp, uint2 *__restrict__ ray_range,
                              uint32_t *__restrict__ counter);
-__global__ void composite_kernel(const uint2 *__restrict__ ray_range, const float4 *__restrict__ so, uint32_t n_rays,
-                                 float t_min, float bg0, float bg1, float bg2, float4 *__restrict__ out);
+__global__ void composite_kernel(CamParams cam, uint32_t ray0, const uint2 *__restrict__ ray_range,
+                                 const float4 *__restrict__ so, uint32_t n_rays, float t_min, float bg0, float bg1,
+                                 float bg2, float4 *__restrict__ out);
 
 // Explicit work buffers of one frame render (the serving loop gives each request its own).
 struct FrameWork {
@@ -112,12 +144,15 @@ nr_status render_rays(const nr_subject *s, const FieldParams &P, const uint32_t 
 nr_status render_frame(const nr_subject *s, const FieldParams &P, const uint32_t *bits, const nr_camera *cam,
                        const nr_render_opts *opts, const FrameWork &w, float4 *dst, cudaStream_t st);
 
-CamParams cam_params(const nr_camera *c);
+// max_slots: the ray numbers that the caller's buffers hold (at least width x height); patch order
+// is taken where its numbers, which cover the image in whole patches, stay within them and within
+// 1/8 over the pixels.
+CamParams cam_params(const nr_camera *c, uint64_t max_slots);
+uint32_t ray_slots(const CamParams &c);                       // ray numbers of an image
 int render_path(const nr_render_opts *o);                     // the launch_field path the options select
 bool path_uses_tcgen05(const nr_render_opts *o, int path);    // needs prepare_t5, sets the error word
 nr_status check_field_timeouts(nr_subject *s, cudaStream_t st);   // NR_ETIMEOUT if a bounded wait gave up
 int num_sms(int device);
-size_t field_f32_smem(const FieldParams &P);
 // mma_path for the bf16/f16 tiers: 0 = the warp-specialised tcgen05 pipeline (field_ws.cu), 1 = tcgen05
 // with one group per tile and activations through shared memory (field_t5.cu), 2 = warp-level mma.sync
 // over two m-tiles per weight read (12 warps/SM), 4 = warp-level mma.sync over one 16-row m-tile per

@@ -120,7 +120,7 @@ extern "C" nr_status nr_render_static(nr_subject *s, const nr_camera *cam, const
   const bool t5 = path_uses_tcgen05(opts, path);
   if (t5 && (r = prepare_t5(s, st)) != NR_OK) return r;
   const FieldParams P = field_params(s, opts);
-  const CamParams C = cam_params(cam);
+  const CamParams C = cam_params(cam, n_rays);   // patches only where they cover the image exactly
   MarchParams mp{};
   for (int k = 0; k < 3; ++k) {
     mp.bmin[k] = s->bmin[k];
@@ -137,8 +137,9 @@ extern "C" nr_status nr_render_static(nr_subject *s, const nr_camera *cam, const
   if ((r = launch_field(P, opts->mlp_dtype, kModeRender, sc->samp, 0, sc->counter, (float *)sc->samp_out, s->device,
                         st, path)) != NR_OK)
     return r;
-  composite_kernel<<<(nr_ + 255) / 256, 256, 0, st>>>(sc->ray_range, sc->samp_out, nr_, opts->t_min, cam->bg[0],
-                                                      cam->bg[1], cam->bg[2], reinterpret_cast<float4 *>(out_rgba));
+  composite_kernel<<<(nr_ + 255) / 256, 256, 0, st>>>(C, 0, sc->ray_range, sc->samp_out, nr_, opts->t_min,
+                                                      cam->bg[0], cam->bg[1], cam->bg[2],
+                                                      reinterpret_cast<float4 *>(out_rgba));
   NR_CHECK_CUDA(cudaGetLastError());
   count_launches(3);
   return t5 ? check_field_timeouts(s, st) : NR_OK;
