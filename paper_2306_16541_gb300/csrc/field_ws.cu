@@ -317,31 +317,41 @@ __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, 
   float *sF8 = reinterpret_cast<float *>(sTmem + 4);   // fp8 tier's table (16-byte aligned)
   constexpr bool F8 = kIsF8<T>;
 
-  {  // a block with no tile leaves before any set-up (the live count is known only here)
-    const uint32_t n0 = n_dev ? *n_dev : n_fixed;
-    if ((uint64_t)blockIdx.x * kWsGroups * 128 >= n0) return;
-  }
+  // The groups' first tiles: a launch with fewer tiles than groups spreads them over the SMs (a tile
+  // alone on its SM does not wait for another's gathers), a larger one gives a block's groups
+  // neighbouring tiles.  A block with no tile leaves before any set-up (the live count is known
+  // only here).
+  const uint32_t n = n_dev ? *n_dev : n_fixed;
+  const uint32_t n_tiles = (n + 127) / 128;
+  const uint32_t tstride = gridDim.x * kWsGroups;
+  const bool spread = n_tiles < tstride;
+  if (spread ? blockIdx.x >= n_tiles : blockIdx.x * kWsGroups >= n_tiles) return;
+  auto first_tile = [&](int g) { return spread ? (uint32_t)g * gridDim.x + blockIdx.x : blockIdx.x * kWsGroups + (uint32_t)g; };
   const int tid = threadIdx.x, warp = tid >> 5;
   const bool res = P.res_enabled != 0;
   const int H = P.hidden;
   const float *sBox = nullptr;
   {  // weights, biases, pose; barriers and the layer table; TMEM
+    // the loads of every part first, so that the set-up waits for memory once (each round of a
+    // frame repeats it)
     const int4 *src = reinterpret_cast<const int4 *>(wblob);
     int4 *dst = reinterpret_cast<int4 *>(sW);
-    for (int i = tid; i < L.total / 16; i += blockDim.x) dst[i] = __ldg(src + i);
-    for (int i = tid; i < n_bt * kWsBiasTile / 16; i += blockDim.x) dst[bt0 / 16 + i] = make_int4(0, 0, 0, 0);
-    auto copyb = [&](int dsto, const float *s, int nv, int npad) {
-      for (int i = tid; i < npad; i += blockDim.x) sBias[dsto + i] = i < nv ? s[i] : 0.f;
-    };
-    copyb(bl.r1, P.bias1, kWidth, kWidth);
-    copyb(bl.r2, P.blob + P.lay.r2b, kWidth, kWidth);
-    copyb(bl.r3, P.blob + P.lay.r3b, kWidth, kWidth);
-    copyb(bl.r4, P.blob + P.lay.r4b, kWidth, kWidth);
-    copyb(bl.r5, P.blob + P.lay.r5b, 3, 4);
-    copyb(bl.c0, P.blob + P.lay.c0b, kWidth, kWidth);
-    for (int l = 0; l < H - 1; ++l) copyb(bl.c0 + kWidth * (l + 1), P.blob + P.lay.chb[l], kWidth, kWidth);
-    copyb(bl.cl, P.blob + P.lay.clb, 4, 4);
-    sBox = stage_pose(P, sG, tid, blockDim.x);
+    float bv[5 + kMaxHidden] = {};   // this column's hidden biases: r1 (pose folded in), r4, r2, r3, c0, ch[]
+    if (!F8 && tid < kWidth) {
+      bv[0] = P.bias1[tid];
+      bv[1] = P.blob[P.lay.r4b + tid];
+      bv[2] = P.blob[P.lay.r2b + tid];
+      bv[3] = P.blob[P.lay.r3b + tid];
+      bv[4] = P.blob[P.lay.c0b + tid];
+#pragma unroll
+      for (int l = 0; l < kMaxHidden - 1; ++l) bv[5 + l] = l < H - 1 ? P.blob[P.lay.chb[l] + tid] : 0.f;
+    }
+    const float ob = tid < 4 ? (tid < 3 ? P.blob[P.lay.r5b + tid] : 0.f) : tid < 8 ? P.blob[P.lay.clb + tid - 4] : 0.f;
+#pragma unroll 8
+    for (int i = tid; i < L.total / 16; i += kWsThreads) dst[i] = __ldg(src + i);
+    for (int i = tid; i < n_bt * kWsBiasTile / 16; i += kWsThreads) dst[bt0 / 16 + i] = make_int4(0, 0, 0, 0);
+    if (tid < 8) sBias[(tid < 4 ? bl.r5 : bl.cl - 4) + tid] = ob;   // the output layers' float32 biases
+    sBox = stage_pose(P, sG, tid, kWsThreads);
     __syncthreads();
     // biases into the B operands: columns 39 and 40 of residual layers 1 (the pose-folded bias)
     // and 4 (its gamma part), columns 0 and 1 of the bias tiles
@@ -378,12 +388,14 @@ __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, 
         *reinterpret_cast<T *>(sW + tile + sw128(n, k)) = hi;
         *reinterpret_cast<T *>(sW + tile + sw128(n, k + 1)) = TcOps<T>::cvt(v - (float)hi);
       };
-      put(L.r1, 39, P.bias1[n]);
-      put(L.r4g, 39, P.blob[P.lay.r4b + n]);
-      put(bt0 + 0 * kWsBiasTile, 0, P.blob[P.lay.r2b + n]);
-      put(bt0 + 1 * kWsBiasTile, 0, P.blob[P.lay.r3b + n]);
-      put(bt0 + 2 * kWsBiasTile, 0, P.blob[P.lay.c0b + n]);
-      for (int l = 0; l < P.hidden - 1; ++l) put(bt0 + (3 + l) * kWsBiasTile, 0, P.blob[P.lay.chb[l] + n]);
+      put(L.r1, 39, bv[0]);
+      put(L.r4g, 39, bv[1]);
+      put(bt0 + 0 * kWsBiasTile, 0, bv[2]);
+      put(bt0 + 1 * kWsBiasTile, 0, bv[3]);
+      put(bt0 + 2 * kWsBiasTile, 0, bv[4]);
+#pragma unroll
+      for (int l = 0; l < kMaxHidden - 1; ++l)
+        if (l < H - 1) put(bt0 + (3 + l) * kWsBiasTile, 0, bv[5 + l]);
     }
     if (tid == 0) {
       for (int g = 0; g < 3 * kWsGroups; ++g)   // input ready: four worker warps; the others: one commit
@@ -430,16 +442,12 @@ __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, 
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
   const uint32_t tmem0 = *sTmem;
-  const uint32_t n = n_dev ? *n_dev : n_fixed;
-  const uint32_t n_tiles = (n + 127) / 128;
-  const uint32_t tstride = gridDim.x * kWsGroups;
-
   if (tid >= kWsWorkers) {
     // ------------------------------------------------------------- issuers
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kWsRegsIssuer));
     const int g = warp - kWsWorkers / 32;
     if ((tid & 31) == 0) {
-      const uint32_t t0 = blockIdx.x * kWsGroups + g;
+      const uint32_t t0 = first_tile(g);
       const uint32_t tiles = t0 < n_tiles ? (n_tiles - t0 + tstride - 1) / tstride : 0u;
       const int n_layers = (res ? 5 : 0) + H + 1;
       ws_issue<F8>(tmem0 + (uint32_t)g * kWsSlotCols, smem_u32(sBar + g), smem_u32(sBar + kWsGroups + g),
@@ -480,7 +488,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, 
     // The inverse-LBS warp of the next tile runs in this tile's MLP waits: its support-box tests
     // in the first wait, one round of four bones in each later one; what is left when the next
     // tile starts is finished then.
-    uint32_t tile = blockIdx.x * kWsGroups + g;
+    uint32_t tile = first_tile(g);
     LbsState nx;
     float d_next = 0.f;
     if (tile < n_tiles) {

@@ -182,13 +182,18 @@ __device__ __forceinline__ LevelCell level_cell(const FieldParams &P, int l, flo
   c.N = P.level_res[l];
   const float fn = (float)c.N;
   const float q0 = p0 * fn, q1 = p1 * fn, q2 = p2 * fn;
-  const float a0 = fminf(floorf(q0), fn - 1.f), a1 = fminf(floorf(q1), fn - 1.f), a2 = fminf(floorf(q2), fn - 1.f);
-  c.f0 = q0 - a0;
-  c.f1 = q1 - a1;
-  c.f2 = q2 - a2;
-  c.i0 = (uint32_t)a0;
-  c.i1 = (uint32_t)a1;
-  c.i2 = (uint32_t)a2;
+  // floor of 0 <= q < 2^23 without a conversion: q + 2^23 rounded down holds the integer in its low
+  // bits (floorf and the float-to-integer conversion run at an eighth of the add's rate)
+  constexpr float kTwo23 = 8388608.f;
+  const float top = (fn - 1.f) + kTwo23;
+  const float t0 = fminf(__fadd_rd(q0, kTwo23), top), t1 = fminf(__fadd_rd(q1, kTwo23), top),
+              t2 = fminf(__fadd_rd(q2, kTwo23), top);
+  c.f0 = q0 - (t0 - kTwo23);
+  c.f1 = q1 - (t1 - kTwo23);
+  c.f2 = q2 - (t2 - kTwo23);
+  c.i0 = __float_as_uint(t0) & 0x7fffffu;
+  c.i1 = __float_as_uint(t1) & 0x7fffffu;
+  c.i2 = __float_as_uint(t2) & 0x7fffffu;
   return c;
 }
 

@@ -88,13 +88,18 @@ __global__ void __launch_bounds__(256) march_kernel(CamParams cam, MarchParams m
 // occ_grid^3 is a multiple of 32, so a warp's tile is one word of the bitfield, written by its
 // ballot.
 //
-// Bound by the FMA pipe (28 K FMAs per sample of the tiny workload) at eight warps an SM: the
-// weights (100-135 KB) and 13.3 KB of activations a warp fill the shared memory.
-constexpr int kF32MaxThreads = 256;
-constexpr int kF32WarpFloats = (kWidth + kTileGamma) * 32;
+// Bound by the FMA pipe (28 K FMAs per sample of the tiny workload) and, level with it, the loads of
+// its operands, at eight warps an SM: the weights (100-135 KB) and 13.3 KB of activations a warp
+// fill the shared memory.  Forming gamma twice instead of holding it makes room for twelve warps,
+// which gained nothing (a 250,007-point query 382 -> 391 us); the density grid, which has no gamma,
+// takes twelve.
+template <int MODE>
+constexpr int kF32MaxThreads = MODE == kModeDensity ? 384 : 256;
+template <int MODE>
+constexpr int kF32WarpFloats = (kWidth + (MODE == kModeDensity ? 0 : kTileGamma)) * 32;
 
 template <int MODE>
-__global__ void __launch_bounds__(kF32MaxThreads, 1) field_f32_kernel(FieldParams P, const float4 *__restrict__ in,
+__global__ void __launch_bounds__(kF32MaxThreads<MODE>, 1) field_f32_kernel(FieldParams P, const float4 *__restrict__ in,
                                                                       uint32_t n_fixed,
                                                                       const uint32_t *__restrict__ n_dev,
                                                                       float *__restrict__ out) {
@@ -103,7 +108,7 @@ __global__ void __launch_bounds__(kF32MaxThreads, 1) field_f32_kernel(FieldParam
   float *sG = sW + P.lay.total;
   float *sB1 = sG + kPoseSmem;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-  float *h = sB1 + kWidth + warp * kF32WarpFloats;   // this warp's activations: 64 rows, then gamma
+  float *h = sB1 + kWidth + warp * kF32WarpFloats<MODE>;   // this warp's activations: 64 rows, then gamma
   float *g = h + kWidth * 32;
   constexpr bool kCells = MODE == kModeDensity || MODE == kModePose;
   const uint32_t n = kCells ? (uint32_t)P.occ_grid * P.occ_grid * P.occ_grid : (n_dev ? *n_dev : n_fixed);
@@ -205,9 +210,9 @@ static size_t f32_base_smem(const FieldParams &P) { return sizeof(float) * (P.la
 template <int MODE>
 static nr_status launch_f32(const FieldParams &P, const float4 *in, uint32_t n_fixed, const uint32_t *n_dev, float *out,
                             int device, cudaStream_t st) {
-  constexpr size_t kSmemMax = 227 * 1024, kWarpBytes = kF32WarpFloats * sizeof(float);
+  constexpr size_t kSmemMax = 227 * 1024, kWarpBytes = kF32WarpFloats<MODE> * sizeof(float);
   const size_t base = f32_base_smem(P);
-  const int warps = (int)std::min<size_t>(kF32MaxThreads / 32, (kSmemMax - base) / kWarpBytes);
+  const int warps = (int)std::min<size_t>(kF32MaxThreads<MODE> / 32, (kSmemMax - base) / kWarpBytes);
   const size_t smem = base + warps * kWarpBytes;
   NR_CHECK_CUDA(cudaFuncSetAttribute(field_f32_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   field_f32_kernel<MODE><<<num_sms(device), 32 * warps, smem, st>>>(P, in, n_fixed, n_dev, out);
@@ -464,9 +469,11 @@ bool path_uses_tcgen05(const nr_render_opts *o, int path) {
 
 nr_status check_field_timeouts(nr_subject *s, cudaStream_t st) {
   if (!s->t5_err) return NR_OK;
-  uint32_t word = 0;
-  NR_CHECK_CUDA(cudaMemcpyAsync(&word, s->t5_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+  // into pinned memory: a copy to the stack goes through the driver's staging buffer
+  if (!s->h_err) NR_CHECK_CUDA(cudaMallocHost((void **)&s->h_err, sizeof(uint32_t)));
+  NR_CHECK_CUDA(cudaMemcpyAsync(s->h_err, s->t5_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   NR_CHECK_CUDA(cudaStreamSynchronize(st));
+  const uint32_t word = *s->h_err;
   if (word == 0) return NR_OK;
   NR_CHECK_CUDA(cudaMemsetAsync(s->t5_err, 0, sizeof(uint32_t), st));
   set_error("field kernel: a bounded wait on the tensor-core pipeline gave up (code %u); the output is invalid",

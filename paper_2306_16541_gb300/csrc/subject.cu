@@ -707,6 +707,7 @@ static void free_subject(nr_subject *s) {
   for (cudaEvent_t &e : s->prof_ev)
     if (e) cudaEventDestroy(e);
   if (s->pose_ev) cudaEventDestroy(s->pose_ev);
+  if (s->h_err) cudaFreeHost(s->h_err);
   s->magic = 0;
   delete s;
 }
