@@ -42,6 +42,7 @@ __global__ void cnn_fc_fwd(const float *__restrict__ W, const float *__restrict_
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= C0) return;
   float a = b[o];
+#pragma unroll 32
   for (int k = 0; k < kCnnZ; ++k) a = fmaf(W[(size_t)o * kCnnZ + k], z[k], a);
   h[o] = leaky(a);
 }
@@ -92,6 +93,70 @@ __global__ void __launch_bounds__(256) cnn_convt_fwd(const float *__restrict__ i
   }
 }
 
+// The same for a layer wide enough to give every thread its own sums (split 1): kFwdOut outputs at
+// one position.  The eight output parities (blockIdx.z) take different taps and one class of a
+// block shares them, so its weights come from shared memory as broadcasts (two 16-byte loads per
+// output and input) and its inputs are read coalesced, once for the kFwdOut outputs; a thread per
+// output read two values from L1 for each multiply-add.  Each sum runs over the inputs and taps in
+// the order of cnn_convt_fwd, so the volume keeps its bits.  0.37 and 0.45 ms for the last two
+// layers before.
+constexpr int kFwdOut = 4, kFwdIn = 16, kFwdThreads = 128;
+__global__ void __launch_bounds__(kFwdThreads) cnn_convt_fwd_wide(const float *__restrict__ in,
+                                                                  const float *__restrict__ W,
+                                                                  const float *__restrict__ b, int Cin, int Cout,
+                                                                  int r, int act, float *__restrict__ out) {
+  __shared__ float4 sw[kFwdIn * kFwdOut * 2];
+  const int par[3] = {(int)(blockIdx.z >> 2), (int)(blockIdx.z >> 1) & 1, (int)blockIdx.z & 1};   // of z, y, x
+  const int r3 = r * r * r, m = blockIdx.x * kFwdThreads + threadIdx.x, o0 = blockIdx.y * kFwdOut;
+  const bool valid = m < r3;
+  const int mx = m % r, my = (m / r) % r, mz = m / (r * r);
+  // tap a of an axis: input m + parity - a, kernel index (parity ? 0 : 1) + 2 a
+  int at[8];
+  bool ok[8];
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    const int z = mz + par[0] - (t >> 2), y = my + par[1] - ((t >> 1) & 1), x = mx + par[2] - (t & 1);
+    ok[t] = valid && z >= 0 && y >= 0 && x >= 0 && z < r && y < r && x < r;
+    at[t] = ok[t] ? (z * r + y) * r + x : 0;
+  }
+  float acc[kFwdOut] = {};
+  for (int i0 = 0; i0 < Cin; i0 += kFwdIn) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < kFwdIn * kFwdOut * 8; e += kFwdThreads) {
+      const int t = e & 7, oc = (e >> 3) % kFwdOut, i = i0 + e / (8 * kFwdOut);
+      const int kz = (par[0] ? 0 : 1) + 2 * (t >> 2), ky = (par[1] ? 0 : 1) + 2 * ((t >> 1) & 1),
+                kx = (par[2] ? 0 : 1) + 2 * (t & 1);
+      reinterpret_cast<float *>(sw)[e] =
+          i < Cin && o0 + oc < Cout ? __ldg(W + ((size_t)i * Cout + o0 + oc) * 64 + (kz * 4 + ky) * 4 + kx) : 0.f;
+    }
+    __syncthreads();
+    const int ni = min(kFwdIn, Cin - i0);
+#pragma unroll 2
+    for (int ic = 0; ic < ni; ++ic) {
+      const float *xi = in + (size_t)(i0 + ic) * r3;
+      float x[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) x[t] = ok[t] ? __ldg(xi + at[t]) : 0.f;
+#pragma unroll
+      for (int oc = 0; oc < kFwdOut; ++oc) {
+        const float4 u = sw[(ic * kFwdOut + oc) * 2], v = sw[(ic * kFwdOut + oc) * 2 + 1];
+        const float w[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int t = 0; t < 8; ++t) acc[oc] = fmaf(x[t], w[t], acc[oc]);
+      }
+    }
+  }
+  if (!valid) return;
+  const int R = 2 * r;
+  const size_t u = ((size_t)(2 * mz + par[0]) * R + 2 * my + par[1]) * R + 2 * mx + par[2];
+#pragma unroll
+  for (int oc = 0; oc < kFwdOut; ++oc)
+    if (o0 + oc < Cout) {
+      const float v = acc[oc] + b[o0 + oc];
+      out[(size_t)(o0 + oc) * R * R * R + u] = act ? leaky(v) : v;
+    }
+}
+
 // W^c[c][v] = softmax_c(logit[c][v] + log_prior[c][v])
 __global__ void cnn_softmax_fwd(const float *__restrict__ logit, const float *__restrict__ log_prior, int V,
                                 float *__restrict__ w) {
@@ -129,78 +194,212 @@ __global__ void cnn_softmax_bwd(const float *__restrict__ w, const float *__rest
   }
 }
 
-// din[i][q] = leaky'(in[i][q]) sum_o sum_k W[i][o][k] dout[o][2 q - 1 + k]: `split` lanes per
-// input (outputs o = j, j + split, ...), summed over shuffles
-__global__ void __launch_bounds__(256) cnn_convt_bwd_data(const float *__restrict__ in, const float *__restrict__ W,
-                                                          const float *__restrict__ dout, int Cin, int Cout, int r,
-                                                          int split, float *__restrict__ din) {
-  const size_t r3 = (size_t)r * r * r;
-  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t idx = t / split;
-  const int j = (int)(t % split);
-  const bool valid = idx < (size_t)Cin * r3;
-  float acc = 0.f;
-  if (valid) {
-    const int q = (int)(idx % r3), i = (int)(idx / r3);
-    const int x = q % r, y = (q / r) % r, zz = q / (r * r);
-    const int R = 2 * r;
-    const size_t R3 = (size_t)R * R * R;
-    for (int o = j; o < Cout; o += split) {
-      const float *wi = W + ((size_t)i * Cout + o) * 64;
-      const float *go = dout + (size_t)o * R3;
-      for (int kz = 0; kz < 4; ++kz) {
-        const int uz = 2 * zz - 1 + kz;
-        if (uz < 0 || uz >= R) continue;
-        for (int ky = 0; ky < 4; ++ky) {
-          const int uy = 2 * y - 1 + ky;
-          if (uy < 0 || uy >= R) continue;
+// din[i][q] = leaky'(in[i][q]) sum_o sum_k W[i][o][k] dout[o][2 q - 1 + k].
+//
+// r >= 8: a block takes 64 positions and four inputs, its four pairs of warps every fourth output;
+// a thread's 64 dout values of an output serve the four inputs, whose weights come from shared
+// memory as broadcasts.  (One group of lanes per input value, each reading its own weight rows and
+// window, took 0.17-0.39 ms a layer.)
+constexpr int kBackIn = 4;
+__global__ void __launch_bounds__(256) cnn_convt_bwd_data_wide(const float *__restrict__ in, const float *__restrict__ W,
+                                                               const float *__restrict__ dout, int Cin, int Cout, int r,
+                                                               float *__restrict__ din) {
+  __shared__ float4 sw[4][kBackIn][16];
+  __shared__ float red[4][kBackIn][64];
+  const int part = threadIdx.x >> 6, p = threadIdx.x & 63, q = blockIdx.x * 64 + p, i0 = blockIdx.y * kBackIn;
+  const int x = q % r, y = (q / r) % r, z = q / (r * r), R = 2 * r;
+  const size_t R3 = (size_t)R * R * R;
+  float acc[kBackIn] = {};
+  for (int o0 = 0; o0 < Cout; o0 += 4) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < 4 * kBackIn * 64; e += 256) {
+      const int k = e & 63, i = i0 + ((e >> 6) % kBackIn), o = o0 + e / (64 * kBackIn);
+      reinterpret_cast<float *>(sw)[e] = i < Cin && o < Cout ? __ldg(W + ((size_t)i * Cout + o) * 64 + k) : 0.f;
+    }
+    __syncthreads();
+    const int o = o0 + part;
+    if (o >= Cout) continue;
+    const float *go = dout + (size_t)o * R3;
 #pragma unroll
-          for (int kx = 0; kx < 4; ++kx) {
-            const int ux = 2 * x - 1 + kx;
-            if (ux < 0 || ux >= R) continue;
-            acc = fmaf(wi[(kz * 4 + ky) * 4 + kx], go[((size_t)uz * R + uy) * R + ux], acc);
-          }
+    for (int kz = 0; kz < 4; ++kz) {
+      const int uz = 2 * z - 1 + kz;
+#pragma unroll
+      for (int ky = 0; ky < 4; ++ky) {
+        const int uy = 2 * y - 1 + ky;
+        const bool row = uz >= 0 && uz < R && uy >= 0 && uy < R;
+        const float *gr = go + ((ptrdiff_t)uz * R + uy) * R;
+        float g[4];
+#pragma unroll
+        for (int kx = 0; kx < 4; ++kx) {
+          const int ux = 2 * x - 1 + kx;
+          g[kx] = row && ux >= 0 && ux < R ? __ldg(gr + ux) : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < kBackIn; ++i) {
+          const float4 w = sw[part][i][kz * 4 + ky];
+          acc[i] = fmaf(w.x, g[0], fmaf(w.y, g[1], fmaf(w.z, g[2], fmaf(w.w, g[3], acc[i]))));
         }
       }
     }
   }
-  for (int off = split >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if (valid && j == 0) din[idx] = acc * leaky_grad(in[idx]);
+#pragma unroll
+  for (int i = 0; i < kBackIn; ++i) red[part][i][p] = acc[i];
+  __syncthreads();
+  const int i = i0 + part;   // pair of warps `part` finishes input i0 + part
+  static_assert(kBackIn == 4, "one input per pair of warps");
+  if (i < Cin) {
+    const size_t at = (size_t)i * r * r * r + q;
+    din[at] = ((red[0][part][p] + red[1][part][p]) + (red[2][part][p] + red[3][part][p])) * leaky_grad(in[at]);
+  }
 }
 
-// dW[i][o][k] = sum_q in[i][q] dout[o][2 q - 1 + k], one thread per weight (k fastest)
-__global__ void __launch_bounds__(256) cnn_convt_bwd_weight(const float *__restrict__ in, const float *__restrict__ dout,
-                                                            int Cin, int Cout, int r, float *__restrict__ dW) {
-  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (size_t)Cin * Cout * 64) return;
-  const int k = (int)(idx % 64);
-  const size_t io = idx / 64;
-  const int o = (int)(io % Cout), i = (int)(io / Cout);
-  const int kx = k & 3, ky = (k >> 2) & 3, kz = k >> 4;
-  const int R = 2 * r;
-  const size_t R3 = (size_t)R * R * R;
+// r = 1, 2, 4: a block takes one input channel with every position in its registers.  Its threads
+// are the 64 taps by four outputs, so the weights, the larger operand here, are read once and
+// coalesced; the outputs' gradients lie in shared memory with a rim of zeros.
+template <int r>
+__global__ void __launch_bounds__(256) cnn_convt_bwd_data_deep(const float *__restrict__ in, const float *__restrict__ W,
+                                                               const float *__restrict__ dout, int Cout,
+                                                               float *__restrict__ din) {
+  constexpr int R = 2 * r, P = R + 2, R3 = R * R * R, P3 = P * P * P, r3 = r * r * r, OCH = r == 4 ? 4 : 16;
+  __shared__ float pad[OCH * P3];
+  __shared__ float red[8][r3];
+  const int i = blockIdx.x, k = threadIdx.x & 63, kx = k & 3, ky = (k >> 2) & 3, kz = k >> 4;
+  const float *Wi = W + (size_t)i * Cout * 64 + k;
+  float acc[r3] = {};
+  for (int o0 = 0; o0 < Cout; o0 += OCH) {
+    float w[OCH / 4];
+#pragma unroll
+    for (int j = 0; j < OCH / 4; ++j) {
+      const int o = o0 + (threadIdx.x >> 6) + 4 * j;
+      w[j] = o < Cout ? __ldg(Wi + (size_t)o * 64) : 0.f;
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < OCH * P3; e += 256) {
+      const int o = o0 + e / P3, c = e % P3, ux = c % P - 1, uy = (c / P) % P - 1, uz = c / (P * P) - 1;
+      pad[e] = o < Cout && ux >= 0 && ux < R && uy >= 0 && uy < R && uz >= 0 && uz < R
+                   ? __ldg(dout + (size_t)o * R3 + (uz * R + uy) * R + ux)
+                   : 0.f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < OCH / 4; ++j) {
+      const float *g = pad + ((threadIdx.x >> 6) + 4 * j) * P3 + (kz * P + ky) * P + kx;
+#pragma unroll
+      for (int q = 0; q < r3; ++q)
+        acc[q] = fmaf(w[j], g[(2 * (q / (r * r)) * P + 2 * ((q / r) % r)) * P + 2 * (q % r)], acc[q]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < r3; ++q) {
+    float v = acc[q];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][q] = v;
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < r3; q += 256) {
+    float v = 0.f;
+#pragma unroll
+    for (int wp = 0; wp < 8; ++wp) v += red[wp][q];
+    din[(size_t)i * r3 + q] = v * leaky_grad(in[(size_t)i * r3 + q]);
+  }
+}
+
+// dW[i][o][k] = sum_q in[i][q] dout[o][2 q - 1 + k].
+//
+// r >= 4: a block takes one output and eight inputs; its threads are the 64 taps by slices of the
+// planes of q.  A dout value serves the eight inputs, whose values are the same for all taps
+// (16-byte broadcasts).  (A thread per weight took 0.43 ms for the last layer's 102,400.)
+constexpr int kWgIn = 8;
+__global__ void __launch_bounds__(512) cnn_convt_bwd_weight_wide(const float *__restrict__ in,
+                                                                 const float *__restrict__ dout, int Cin, int Cout,
+                                                                 int r, int aligned, float *__restrict__ dW) {
+  __shared__ float red[8][kWgIn][64];
+  const int k = threadIdx.x & 63, slice = threadIdx.x >> 6, slices = blockDim.x >> 6;
+  const int kx = k & 3, ky = (k >> 2) & 3, kz = k >> 4, o = blockIdx.x, i0 = blockIdx.y * kWgIn, R = 2 * r;
+  const size_t r3 = (size_t)r * r * r;
+  const float *go = dout + (size_t)o * R * R * R;
+  float acc[kWgIn] = {};
+  for (int z = slice; z < r; z += slices) {
+    const int uz = 2 * z - 1 + kz;
+    if (uz < 0 || uz >= R) continue;
+    for (int y = 0; y < r; ++y) {
+      const int uy = 2 * y - 1 + ky;
+      const bool row = uy >= 0 && uy < R;
+      const float *gr = go + ((ptrdiff_t)uz * R + uy) * R;
+      for (int x = 0; x < r; x += 4) {
+        float g[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int ux = 2 * (x + e) - 1 + kx;
+          g[e] = row && ux >= 0 && ux < R ? __ldg(gr + ux) : 0.f;
+        }
+        const float *xi = in + (size_t)i0 * r3 + (z * r + y) * r + x;
+#pragma unroll
+        for (int i = 0; i < kWgIn; ++i) {
+          if (i0 + i >= Cin) break;
+          float4 v;
+          if (aligned) {
+            v = __ldg(reinterpret_cast<const float4 *>(xi + i * r3));
+          } else {
+            v = make_float4(__ldg(xi + i * r3), __ldg(xi + i * r3 + 1), __ldg(xi + i * r3 + 2), __ldg(xi + i * r3 + 3));
+          }
+          acc[i] = fmaf(v.x, g[0], fmaf(v.y, g[1], fmaf(v.z, g[2], fmaf(v.w, g[3], acc[i]))));
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < kWgIn; ++i) red[slice][i][k] = acc[i];
+  __syncthreads();
+  for (int e = threadIdx.x; e < kWgIn * 64; e += blockDim.x) {
+    const int i = e >> 6;
+    if (i0 + i >= Cin) break;
+    float v = 0.f;
+    for (int sl = 0; sl < slices; ++sl) v += red[sl][i][e & 63];
+    dW[((size_t)(i0 + i) * Cout + o) * 64 + (e & 63)] = v;
+  }
+}
+
+// r = 1, 2: few positions and many weights, so the kernel is the store of dW: a thread per tap
+// row of an output (four weights), a grid row per input, no division.
+__global__ void __launch_bounds__(256) cnn_convt_bwd_weight_deep(const float *__restrict__ in,
+                                                                 const float *__restrict__ dout, int Cout, int r,
+                                                                 int aligned, float *__restrict__ dW) {
+  const int t = blockIdx.x * 256 + threadIdx.x, o = t >> 4, ky = t & 3, kz = (t >> 2) & 3, i = blockIdx.y, R = 2 * r;
+  if (o >= Cout) return;
   const float *xi = in + (size_t)i * r * r * r;
-  const float *go = dout + (size_t)o * R3;
-  float acc = 0.f;
-  for (int zz = 0; zz < r; ++zz) {
-    const int uz = 2 * zz - 1 + kz;
+  const float *go = dout + (size_t)o * R * R * R;
+  float acc[4] = {};
+  for (int z = 0; z < r; ++z) {
+    const int uz = 2 * z - 1 + kz;
     if (uz < 0 || uz >= R) continue;
     for (int y = 0; y < r; ++y) {
       const int uy = 2 * y - 1 + ky;
       if (uy < 0 || uy >= R) continue;
       for (int x = 0; x < r; ++x) {
-        const int ux = 2 * x - 1 + kx;
-        if (ux < 0 || ux >= R) continue;
-        acc = fmaf(xi[((size_t)zz * r + y) * r + x], go[((size_t)uz * R + uy) * R + ux], acc);
+        const float v = __ldg(xi + (z * r + y) * r + x);
+#pragma unroll
+        for (int kx = 0; kx < 4; ++kx) {
+          const int ux = 2 * x - 1 + kx;
+          if (ux >= 0 && ux < R) acc[kx] = fmaf(v, __ldg(go + (uz * R + uy) * R + ux), acc[kx]);
+        }
       }
     }
   }
-  dW[idx] = acc;
+  float *d = dW + ((size_t)i * Cout + o) * 64 + (kz * 4 + ky) * 4;
+  if (aligned) {
+    *reinterpret_cast<float4 *>(d) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+  } else {
+#pragma unroll
+    for (int kx = 0; kx < 4; ++kx) d[kx] = acc[kx];
+  }
 }
 
-// db[o] = sum_u dout[o][u]: one block per channel
-__global__ void cnn_bias_grad(const float *__restrict__ dout, int n_per, float *__restrict__ db) {
-  __shared__ float red[256];
+// db[o] = sum_u dout[o][u]: one block per channel (up to 1024 threads)
+__global__ void __launch_bounds__(1024) cnn_bias_grad(const float *__restrict__ dout, int n_per,
+                                                      float *__restrict__ db) {
+  __shared__ float red[1024];
   const int o = blockIdx.x;
   float a = 0.f;
   for (int u = threadIdx.x; u < n_per; u += blockDim.x) a += dout[(size_t)o * n_per + u];
@@ -285,6 +484,13 @@ nr_status cnn_forward(nr_subject *s, cudaStream_t st) {
     const size_t R = 2 * (size_t)L.r[k];
     const size_t nout = (size_t)L.cout[k] * R * R * R;
     const int sp = cnn_split(nout, L.cin[k]);
+    if (sp == 1) {   // enough outputs for a thread to own whole sums
+      const int r3 = L.r[k] * L.r[k] * L.r[k];
+      cnn_convt_fwd_wide<<<dim3((r3 + kFwdThreads - 1) / kFwdThreads, (L.cout[k] + kFwdOut - 1) / kFwdOut, 8),
+                           kFwdThreads, 0, st>>>(A + L.act[k - 1], s->cnn + L.w[k], s->cnn + L.b[k], L.cin[k],
+                                                 L.cout[k], L.r[k], k < 5 ? 1 : 0, A + L.act[k]);
+      continue;
+    }
     cnn_convt_fwd<<<blocks_for(nout * sp), 256, 0, st>>>(A + L.act[k - 1], s->cnn + L.w[k], s->cnn + L.b[k],
                                                          L.cin[k], L.cout[k], L.r[k], k < 5 ? 1 : 0, sp,
                                                          A + L.act[k]);
@@ -308,13 +514,25 @@ nr_status cnn_backward(nr_subject *s, cudaStream_t st) {
   for (int k = 5; k >= 1; --k) {
     const size_t R = 2 * (size_t)L.r[k];
     const size_t nout = R * R * R;
-    cnn_convt_bwd_weight<<<blocks_for((size_t)L.cin[k] * L.cout[k] * 64), 256, 0, st>>>(
-        A + L.act[k - 1], d0, L.cin[k], L.cout[k], L.r[k], s->g_cnn + L.w[k]);
-    cnn_bias_grad<<<L.cout[k], 256, 0, st>>>(d0, (int)nout, s->g_cnn + L.b[k]);
-    const size_t nin = (size_t)L.cin[k] * L.r[k] * L.r[k] * L.r[k];
-    const int sp = cnn_split(nin, L.cout[k]);
-    cnn_convt_bwd_data<<<blocks_for(nin * sp), 256, 0, st>>>(A + L.act[k - 1], s->cnn + L.w[k], d0, L.cin[k],
-                                                             L.cout[k], L.r[k], sp, d1);
+    const float *x = A + L.act[k - 1], *w = s->cnn + L.w[k];
+    float *gw = s->g_cnn + L.w[k];
+    const int r = L.r[k], cin = L.cin[k], cout = L.cout[k];
+    if (r >= 4)
+      cnn_convt_bwd_weight_wide<<<dim3(cout, (cin + kWgIn - 1) / kWgIn), 64 * std::min(r, 8), 0, st>>>(
+          x, d0, cin, cout, r, ((uintptr_t)x & 15) == 0, gw);
+    else
+      cnn_convt_bwd_weight_deep<<<dim3((cout * 16 + 255) / 256, cin), 256, 0, st>>>(x, d0, cout, r,
+                                                                                    ((uintptr_t)gw & 15) == 0, gw);
+    cnn_bias_grad<<<cout, nout >= 4096 ? 1024 : 256, 0, st>>>(d0, (int)nout, s->g_cnn + L.b[k]);
+    if (r >= 8)
+      cnn_convt_bwd_data_wide<<<dim3(r * r * r / 64, (cin + kBackIn - 1) / kBackIn), 256, 0, st>>>(x, w, d0, cin, cout,
+                                                                                                  r, d1);
+    else if (r == 4)
+      cnn_convt_bwd_data_deep<4><<<cin, 256, 0, st>>>(x, w, d0, cout, d1);
+    else if (r == 2)
+      cnn_convt_bwd_data_deep<2><<<cin, 256, 0, st>>>(x, w, d0, cout, d1);
+    else
+      cnn_convt_bwd_data_deep<1><<<cin, 256, 0, st>>>(x, w, d0, cout, d1);
     std::swap(d0, d1);
     launched += 3;
   }
