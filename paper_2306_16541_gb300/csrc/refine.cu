@@ -169,32 +169,56 @@ struct RefShared {
   double AR[kBones][9], At[kBones][3];    // world rotation and position of each joint
 };
 
+// One layer of MLP_theta, y_t = b_t + sum_k W[t][k] x[k] in increasing k for the unit t of each
+// thread: W passes through shared memory kRefCols columns at a time, read along its rows by the
+// whole block, the next columns in registers meanwhile.  (A thread reading its own row met L2's
+// latency every few values: 0.168 ms for the five layers.)
+constexpr int kRefCols = 16;
+__device__ __forceinline__ float refine_layer(const float *__restrict__ W, const float *__restrict__ b, int out, int in,
+                                              const float *x, float (*sw)[kRefCols + 1]) {
+  constexpr int kPer = kRefCols;   // 256 rows x kRefCols columns by 256 threads
+  const int t = threadIdx.x, c = t % kRefCols, r0 = t / kRefCols;
+  float nx[kPer];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+      const int row = r0 + e * (kRefThreads / kRefCols);
+      nx[e] = row < out && k0 + c < in ? __ldg(W + (size_t)row * in + k0 + c) : 0.f;
+    }
+  };
+  float a = t < out ? b[t] : 0.f;
+  load(0);
+  for (int k0 = 0; k0 < in; k0 += kRefCols) {
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) sw[r0 + e * (kRefThreads / kRefCols)][c] = nx[e];
+    __syncthreads();
+    if (k0 + kRefCols < in) load(k0 + kRefCols);
+    const int n = min(kRefCols, in - k0);
+    for (int k = 0; k < n; ++k) a = fmaf(sw[t][k], x[k0 + k], a);
+  }
+  return a;
+}
+
 // MLP_theta forward, refined rotations and the kinematic chain of pose `om`
 // (72 angles) with root translation `rt`.  Every thread of the block calls it.
 __device__ void refine_forward(const RefParams &P, const float *om, const float *rt, RefShared &sh) {
+  __shared__ float sw[kRefThreads][kRefCols + 1];
   const int t = threadIdx.x;
   if (t < kRefIn) sh.in[t] = om[3 + t];
-  __syncthreads();
   const float *w = P.w;
   int in = kRefIn;
   const float *src = sh.in;
-  for (int l = 0; l < P.layers; ++l) {
-    const float *W = w, *b = w + (size_t)P.width * in;
-    if (t < P.width) {
-      float a = b[t];
-      for (int k = 0; k < in; ++k) a = fmaf(W[(size_t)t * in + k], src[k], a);
-      sh.h[l][t] = fmaxf(a, 0.f);
-    }
-    __syncthreads();
-    w = b + P.width;
+  for (int l = 0; l < P.layers; ++l) {   // refine_layer's barriers order src's writes before its reads
+    const float a = refine_layer(w, w + (size_t)P.width * in, P.width, in, src, sw);
+    if (t < P.width) sh.h[l][t] = fmaxf(a, 0.f);
+    w += (size_t)P.width * in + P.width;
     in = P.width;
     src = sh.h[l];
   }
-  if (t < kRefIn) {
-    const float *W = w, *b = w + (size_t)kRefIn * in;
-    float a = b[t];
-    for (int k = 0; k < in; ++k) a = fmaf(W[(size_t)t * in + k], src[k], a);
-    sh.delta[t] = a;
+  {
+    const float a = refine_layer(w, w + (size_t)kRefIn * in, kRefIn, in, src, sw);
+    if (t < kRefIn) sh.delta[t] = a;
   }
   __syncthreads();
   if (t < kBones) {
@@ -209,20 +233,27 @@ __device__ void refine_forward(const RefParams &P, const float *om, const float 
     }
   }
   __syncthreads();
-  if (t == 0) {
+  if (t < 32) {   // one warp: lanes 0..8 the entries of A_i's rotation, 9..11 its position
+    const int r = t < 9 ? t / 3 : t - 9, c = t % 3;
     for (int i = 0; i < kBones; ++i) {
       const int p = P.parents[i];
-      if (p < 0) {
-        for (int e = 0; e < 9; ++e) sh.AR[i][e] = sh.Rl[i][e];
-        for (int r = 0; r < 3; ++r) sh.At[i][r] = P.J[3 * i + r] + (double)rt[r];
-      } else {
-        mat3_mul(sh.AR[p], sh.Rl[i], sh.AR[i]);
-        for (int r = 0; r < 3; ++r) {
+      if (t < 9) {
+        if (p < 0) {
+          sh.AR[i][t] = sh.Rl[i][t];
+        } else {
+          const double *a = sh.AR[p], *b = sh.Rl[i];
+          sh.AR[i][t] = a[3 * r] * b[c] + a[3 * r + 1] * b[3 + c] + a[3 * r + 2] * b[6 + c];
+        }
+      } else if (t < 12) {
+        if (p < 0) {
+          sh.At[i][r] = P.J[3 * i + r] + (double)rt[r];
+        } else {
           double a = sh.At[p][r];
           for (int m = 0; m < 3; ++m) a += sh.AR[p][3 * r + m] * (P.J[3 * i + m] - P.J[3 * p + m]);
           sh.At[i][r] = a;
         }
       }
+      __syncwarp();
     }
   }
   __syncthreads();
@@ -264,6 +295,14 @@ __global__ void __launch_bounds__(kRefThreads) refine_fk_kernel(RefParams P, con
       g[4 * r + 3] = (float)tr;
     }
   }
+}
+
+// g[j][k] += d[j] x[k] (rows x cols, cols <= the block's threads): a thread keeps its column.
+__device__ __forceinline__ void outer_add(float *__restrict__ g, const float *d, int rows, const float *x, int cols) {
+  const int per = kRefThreads / cols, r0 = threadIdx.x / cols, c = threadIdx.x - r0 * cols;
+  if (r0 >= per) return;
+  const float xc = x[c];
+  for (int j = r0; j < rows; j += per) atomicAdd(g + (size_t)j * cols + c, d[j] * xc);
 }
 
 // From dL/dG [F][24][12] of each pose to dL/d theta (added into g with atomics).
@@ -375,12 +414,13 @@ __global__ void __launch_bounds__(kRefThreads) refine_bwd_kernel(RefParams P, co
   {
     const float *h = sh.h[P.layers - 1];
     float *gW = g + off[P.layers], *gb = gW + (size_t)kRefIn * W;
-    for (int e = t; e < kRefIn * W; e += blockDim.x) atomicAdd(gW + e, dout[e / W] * h[e % W]);
+    outer_add(gW, dout, kRefIn, h, W);
     if (t < kRefIn) atomicAdd(gb + t, dout[t]);
     if (t < W) {
       const float *Wo = P.w + off[P.layers];
       float a = 0.f;
-      for (int j = 0; j < kRefIn; ++j) a = fmaf(Wo[(size_t)j * W + t], dout[j], a);
+#pragma unroll 16
+      for (int j = 0; j < kRefIn; ++j) a = fmaf(__ldg(Wo + (size_t)j * W + t), dout[j], a);
       dcur[t] = h[t] > 0.f ? a : 0.f;
     }
   }
@@ -389,13 +429,14 @@ __global__ void __launch_bounds__(kRefThreads) refine_bwd_kernel(RefParams P, co
     const int in = l == 0 ? kRefIn : W;
     const float *src = l == 0 ? sh.in : sh.h[l - 1];
     float *gW = g + off[l], *gb = gW + (size_t)W * in;
-    for (int e = t; e < W * in; e += blockDim.x) atomicAdd(gW + e, dcur[e / in] * src[e % in]);
+    outer_add(gW, dcur, W, src, in);
     if (t < W) atomicAdd(gb + t, dcur[t]);
     if (l > 0) {
       if (t < W) {
         const float *Wl = P.w + off[l];
         float a = 0.f;
-        for (int j = 0; j < W; ++j) a = fmaf(Wl[(size_t)j * in + t], dcur[j], a);
+#pragma unroll 16
+        for (int j = 0; j < W; ++j) a = fmaf(__ldg(Wl + (size_t)j * in + t), dcur[j], a);
         dnext[t] = sh.h[l - 1][t] > 0.f ? a : 0.f;
       }
       __syncthreads();
