@@ -14,6 +14,11 @@ namespace nr {
 // i of the canonical weight volume (vertices on the box corners, a corner
 // outside the grid contributes zero).  The denominator S is floored at kEpsW.
 
+// A fraction in a cell is formed as __fsub_rn(u, floor(u)) throughout: u is a product, and a
+// compiler free to fuse the two into one multiply-add does so in some kernels (or in one of two
+// copies within a kernel) and not in others, which moves the last bit and, in training, the side
+// of a kink that a sample falls on.
+//
 // Trilinear sample of one bone channel through its corner-block copy: entry
 // (z, y, x), z in [-1, R], y and x in [-1, R-1], holds the float4
 // (V[z][y][x], V[z][y][x+1], V[z][y+1][x], V[z][y+1][x+1]) with V = 0 outside the
@@ -24,7 +29,7 @@ __device__ __forceinline__ float trilinear_quad(const float4 *__restrict__ q, in
   const float fx0 = floorf(ux), fy0 = floorf(uy), fz0 = floorf(uz);
   const int ix = (int)fx0, iy = (int)fy0, iz = (int)fz0;
   if (ix < -1 || iy < -1 || iz < -1 || ix >= R || iy >= R || iz >= R) return 0.f;
-  const float fx = ux - fx0, fy = uy - fy0, fz = uz - fz0;
+  const float fx = __fsub_rn(ux, fx0), fy = __fsub_rn(uy, fy0), fz = __fsub_rn(uz, fz0);
   const int R1 = R + 1;
   const int b = ((iz + 1) * R1 + (iy + 1)) * R1 + (ix + 1);
   const float4 a = __ldg(q + b), c = __ldg(q + b + R1 * R1);
@@ -42,7 +47,7 @@ __device__ __forceinline__ float trilinear_quad_grad(const float4 *__restrict__ 
   const float fx0 = floorf(ux), fy0 = floorf(uy), fz0 = floorf(uz);
   const int ix = (int)fx0, iy = (int)fy0, iz = (int)fz0;
   if (ix < -1 || iy < -1 || iz < -1 || ix >= R || iy >= R || iz >= R) return 0.f;
-  const float fx = ux - fx0, fy = uy - fy0, fz = uz - fz0;
+  const float fx = __fsub_rn(ux, fx0), fy = __fsub_rn(uy, fy0), fz = __fsub_rn(uz, fz0);
   const int R1 = R + 1;
   const int b = ((iz + 1) * R1 + (iy + 1)) * R1 + (ix + 1);
   const float4 a = __ldg(q + b), c = __ldg(q + b + R1 * R1);
@@ -164,7 +169,7 @@ __device__ __forceinline__ void hash_cell(const FieldParams &P, int l, float p0,
   const float fn = (float)N;
   const float q0 = p0 * fn, q1 = p1 * fn, q2 = p2 * fn;
   const float a0 = fminf(floorf(q0), fn - 1.f), a1 = fminf(floorf(q1), fn - 1.f), a2 = fminf(floorf(q2), fn - 1.f);
-  const float f0 = q0 - a0, f1 = q1 - a1, f2 = q2 - a2;
+  const float f0 = __fsub_rn(q0, a0), f1 = __fsub_rn(q1, a1), f2 = __fsub_rn(q2, a2);
   const uint32_t i0 = (uint32_t)a0, i1 = (uint32_t)a1, i2 = (uint32_t)a2;
   const bool dense = (P.dense_mask >> l) & 1u;
 #pragma unroll
@@ -201,7 +206,7 @@ __device__ __forceinline__ void hash_level(const FieldParams &P, int l, float p0
     const float fn = (float)N;
     const float q0 = p0 * fn, q1 = p1 * fn, q2 = p2 * fn;
     const float a0 = fminf(floorf(q0), fn - 1.f), a1 = fminf(floorf(q1), fn - 1.f), a2 = fminf(floorf(q2), fn - 1.f);
-    const float f0 = q0 - a0, f1 = q1 - a1, f2 = q2 - a2;
+    const float f0 = __fsub_rn(q0, a0), f1 = __fsub_rn(q1, a1), f2 = __fsub_rn(q2, a2);
     const uint4 *Q = P.dense_quad + P.dq_off[l] + ((size_t)a2 * N + (uint32_t)a1) * N + (uint32_t)a0;
     const uint4 lo = __ldg(Q), hi = __ldg(Q + (size_t)N * N);
     const uint32_t u[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};

@@ -143,9 +143,9 @@ __device__ __forceinline__ void lbs_round(const FieldParams &P, const float *__r
     const float fx0 = floorf(ux), fy0 = floorf(uy), fz0 = floorf(uz);
     const int ix = (int)fx0, iy = (int)fy0, iz = (int)fz0;
     inb[k] = keep[k] && !(ix < -1 || iy < -1 || iz < -1 || ix >= R || iy >= R || iz >= R);
-    fx[k] = ux - fx0;
-    fy[k] = uy - fy0;
-    fz[k] = uz - fz0;
+    fx[k] = __fsub_rn(ux, fx0);
+    fy[k] = __fsub_rn(uy, fy0);
+    fz[k] = __fsub_rn(uz, fz0);
     const float4 *q = P.wquad + (size_t)i * QC + (inb[k] ? ((iz + 1) * R1 + (iy + 1)) * R1 + (ix + 1) : 0);
     qa[k] = inb[k] ? __ldg(q) : make_float4(0.f, 0.f, 0.f, 0.f);
     qc[k] = inb[k] ? __ldg(q + R1 * R1) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -188,9 +188,9 @@ __device__ __forceinline__ LevelCell level_cell(const FieldParams &P, int l, flo
   const float top = (fn - 1.f) + kTwo23;
   const float t0 = fminf(__fadd_rd(q0, kTwo23), top), t1 = fminf(__fadd_rd(q1, kTwo23), top),
               t2 = fminf(__fadd_rd(q2, kTwo23), top);
-  c.f0 = q0 - (t0 - kTwo23);
-  c.f1 = q1 - (t1 - kTwo23);
-  c.f2 = q2 - (t2 - kTwo23);
+  c.f0 = __fsub_rn(q0, t0 - kTwo23);
+  c.f1 = __fsub_rn(q1, t1 - kTwo23);
+  c.f2 = __fsub_rn(q2, t2 - kTwo23);
   c.i0 = __float_as_uint(t0) & 0x7fffffu;
   c.i1 = __float_as_uint(t1) & 0x7fffffu;
   c.i2 = __float_as_uint(t2) & 0x7fffffu;

@@ -733,7 +733,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams
         const float q0 = p0 * fn, q1 = p1 * fn, q2 = p2 * fn;
         const float a0 = fminf(floorf(q0), fn - 1.f), a1 = fminf(floorf(q1), fn - 1.f),
                     a2 = fminf(floorf(q2), fn - 1.f);
-        const float fr[3] = {q0 - a0, q1 - a1, q2 - a2};
+        const float fr[3] = {__fsub_rn(q0, a0), __fsub_rn(q1, a1), __fsub_rn(q2, a2)};
         HashCell c;
         hash_cell(P, l, p0, p1, p2, c);
         float2 tv[8];   // the corners, loaded before the exchange below
@@ -909,7 +909,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams
                               fz0 < (float)R;
         const bool valid = active && dw != 0.f && in_range;
         const int ix = valid ? (int)fx0 : 0, iy = valid ? (int)fy0 : 0, iz = valid ? (int)fz0 : 0;
-        const float fx = ux - fx0, fy = uy - fy0, fz = uz - fz0;
+        const float fx = __fsub_rn(ux, fx0), fy = __fsub_rn(uy, fy0), fz = __fsub_rn(uz, fz0);
         float v[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c)
