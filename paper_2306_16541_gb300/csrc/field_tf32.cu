@@ -58,6 +58,12 @@ __global__ void __launch_bounds__(kTf32Threads, 1) field_tf32_kernel(FieldParams
     float s0, s1, s2, S;
     lbs_warp(P, sG, x0, x1, x2, s0, s1, s2, S, sBox);
     float f0 = s0, f1 = s1, f2 = s2;
+    if (MODE == kModeRender && !__any_sync(0xffffffffu, valid && S != 0.f)) {
+      // no bone reaches any of the tile's samples: S = 0, alpha = (..) min(S, 1) = 0, and they add
+      // nothing to their rays
+      if (valid) reinterpret_cast<float4 *>(out)[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      continue;
+    }
     float c[2][8][4], o[4];
     if (P.res_enabled) {
       pos_enc(P, s0, s1, s2, put);

@@ -62,6 +62,8 @@ constexpr unsigned long long kWsTimeoutNs = 500000000ull;
 constexpr int kWsF8Bias = (kWsMaxLayers + 3) & ~3;
 constexpr int kWsF8Inv = kWsF8Bias + kWsMaxLayers * 64;
 
+constexpr int kWsBarWords = 3 * kWsGroups + (kWsGroups + 1) / 2;   // 64-bit words: barriers, then ws_last
+
 // One layer as the issuing thread sends it: nk K-steps of A (TMEM column a_col) x B (weights at
 // byte offset b_off of the shared blob), then nk2 K-steps of a second pair into the same
 // accumulator (residual layer 4: [h3 | gamma]).
@@ -194,6 +196,22 @@ __device__ __forceinline__ void tm_st1(uint32_t taddr, uint32_t v) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(v));
 }
 
+// Whether the predicate holds for any thread of worker group g.  Every thread of the group calls it.
+__device__ __forceinline__ bool group_any(int g, bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.or.pred q, %2, 128, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)v), "r"(g + 1)
+      : "memory");
+  return r != 0;
+}
+
+// Per group: its workers have started their last layer (SKIP), behind the barriers.
+__device__ __forceinline__ volatile uint32_t *ws_last(uint64_t *sBar) {
+  return reinterpret_cast<volatile uint32_t *>(sBar + 3 * kWsGroups);
+}
+
 struct WsGroup {
   uint32_t a_bar;       // the group's "input ready" mbarrier (one arrive per worker warp)
   uint32_t d_bar;       // the group's "layer done" mbarrier (the issuer's commit)
@@ -219,19 +237,21 @@ __device__ __forceinline__ void ws_layer(const WsGroup &G, uint32_t &phase, bool
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// The issuer of one group: for each of its n layer steps, wait (bounded) for the group's input,
-// send the layer's MMAs and commit them; then commit once more and wait until every MMA it issued
-// has completed.  One thread.
-template <bool F8>
+// The issuer of one group: for each of the layer steps that its workers start, wait (bounded) for
+// the group's input, send the layer's MMAs and commit them, until the workers have set *last (they
+// arrive once more with it) or all n_steps are sent; then commit once more and wait until every MMA
+// it issued has completed.  One thread.
+template <bool F8, bool SKIP>
 __device__ __forceinline__ void ws_issue(uint32_t slot, uint32_t a_bar, uint32_t d_bar, uint32_t drain,
                                          const WsLayer *__restrict__ lay, int n_layers, uint32_t n_steps,
-                                         const uint8_t *sW, uint32_t *err) {
+                                         const uint8_t *sW, const volatile uint32_t *last, uint32_t *err) {
   uint32_t phase = 0;
   for (uint32_t i = 0; i < n_steps; ++i) {
     if (!mbar_wait_bounded(a_bar, phase)) {
       atomicExch(err, 2u);
       break;
     }
+    if (SKIP && *last) break;
     phase ^= 1u;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const WsLayer &Ly = lay[i % (uint32_t)n_layers];
@@ -297,7 +317,10 @@ __device__ __forceinline__ void ws_relu_layer_f8(uint32_t my, float m, const flo
   }
 }
 
-template <typename T, int MODE>
+// SKIP: tiles whose samples no bone reaches skip both MLPs (see below).  For launches without
+// occupancy, where most of the box is such tiles (1920 x 1080 x 192 in fp8: 51.6 -> 26.6 ms); an
+// occupancy grid has dropped those samples already, and the group's vote costs 5 % of a frame.
+template <typename T, int MODE, bool SKIP>
 __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, const uint8_t *__restrict__ wblob,
                                                                  const float4 *__restrict__ in, uint32_t n_fixed,
                                                                  const uint32_t *__restrict__ n_dev,
@@ -312,7 +335,7 @@ __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, 
   float *sBias = reinterpret_cast<float *>(sW + bt0 + n_bt * kWsBiasTile);
   float *sG = sBias + ((bl.total + 3) & ~3);
   uint64_t *sBar = reinterpret_cast<uint64_t *>(sG + kPoseSmem);         // input ready[G], done[G], drain[G]
-  WsLayer *sLay = reinterpret_cast<WsLayer *>(sBar + 3 * kWsGroups);
+  WsLayer *sLay = reinterpret_cast<WsLayer *>(sBar + kWsBarWords);
   uint32_t *sTmem = reinterpret_cast<uint32_t *>(sLay + kWsMaxLayers);
   float *sF8 = reinterpret_cast<float *>(sTmem + 4);   // fp8 tier's table (16-byte aligned)
   constexpr bool F8 = kIsF8<T>;
@@ -397,6 +420,9 @@ __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, 
       for (int l = 0; l < kMaxHidden - 1; ++l)
         if (l < H - 1) put(bt0 + (3 + l) * kWsBiasTile, 0, bv[5 + l]);
     }
+    if constexpr (SKIP) {
+      if (tid < kWsGroups) ws_last(sBar)[tid] = 0u;
+    }
     if (tid == 0) {
       for (int g = 0; g < 3 * kWsGroups; ++g)   // input ready: four worker warps; the others: one commit
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(sBar + g)), "r"(g < kWsGroups ? 4 : 1));
@@ -450,8 +476,9 @@ __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, 
       const uint32_t t0 = first_tile(g);
       const uint32_t tiles = t0 < n_tiles ? (n_tiles - t0 + tstride - 1) / tstride : 0u;
       const int n_layers = (res ? 5 : 0) + H + 1;
-      ws_issue<F8>(tmem0 + (uint32_t)g * kWsSlotCols, smem_u32(sBar + g), smem_u32(sBar + kWsGroups + g),
-               smem_u32(sBar + 2 * kWsGroups + g), sLay, n_layers, tiles * (uint32_t)n_layers, sW, err);
+      ws_issue<F8, SKIP>(tmem0 + (uint32_t)g * kWsSlotCols, smem_u32(sBar + g), smem_u32(sBar + kWsGroups + g),
+               smem_u32(sBar + 2 * kWsGroups + g), sLay, n_layers, tiles * (uint32_t)n_layers, sW,
+               SKIP ? ws_last(sBar) + g : nullptr, err);
     }
     __syncwarp();
   } else {
@@ -509,6 +536,16 @@ __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, 
       }
       const bool more = tile + tstride < n_tiles;
       if (more) load_in(tile + tstride, nx, d_next);
+      if constexpr (SKIP) {
+        // A sample that no bone reaches has S = 0, hence alpha = (..) min(S, 1) = 0, and adds
+        // nothing to its ray.  A tile of such samples (in step order a few neighbouring rays at one
+        // depth, so most of the box away from the body) skips both MLPs.
+        if (!group_any(g, valid && S != 0.f)) {
+          if (valid) reinterpret_cast<float4 *>(out)[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (more) lbs_begin(P, sG, sBox, nx, nx_valid);
+          continue;
+        }
+      }
       int stage = 0;
       auto overlap = [&]() {
         if (!more) return;
@@ -669,6 +706,15 @@ __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, 
         }
       }
     }
+    // SKIP: release the issuer from its next wait (unless a wait of this warp gave up: it has stopped
+    // arriving, and the issuer's own wait ends by its bound)
+    if constexpr (SKIP) {
+      __syncwarp();
+      if ((tid & 31) == 0 && ok) {
+        ws_last(sBar)[g] = 1u;
+        mbar_arrive(G.a_bar);
+      }
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -683,19 +729,28 @@ static size_t ws_smem(int hidden) {
   const TcBias bl = tc_bias_layout(hidden);
   size_t b = 1024 + (size_t)((L.total + 1023) & ~1023) + (size_t)(hidden + 2) * kWsBiasTile;
   b += sizeof(float) * (((bl.total + 3) & ~3) + kPoseSmem);
-  b += sizeof(uint64_t) * (3 * kWsGroups) + sizeof(WsLayer) * kWsMaxLayers + 16;
+  b += sizeof(uint64_t) * kWsBarWords + sizeof(WsLayer) * kWsMaxLayers + 16;
   b += sizeof(float) * (kWsF8Inv + 4);               // the fp8 tier's m', b' and input scales
   return b;
+}
+
+template <typename T, int MODE, bool SKIP>
+static nr_status launch_ws_kernel(const FieldParams &P, const uint8_t *blob, const float4 *in, uint32_t n_fixed,
+                                  const uint32_t *n_dev, float *out, uint32_t *err, int device, cudaStream_t st) {
+  const size_t smem = ws_smem(P.hidden);
+  NR_CHECK_CUDA(
+      cudaFuncSetAttribute(field_ws_kernel<T, MODE, SKIP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  field_ws_kernel<T, MODE, SKIP><<<num_sms(device), kWsThreads, smem, st>>>(P, blob, in, n_fixed, n_dev, out, err);
+  NR_CHECK_CUDA(cudaGetLastError());
+  return NR_OK;
 }
 
 template <typename T, int MODE>
 static nr_status launch_ws_mode(const FieldParams &P, const uint8_t *blob, const float4 *in, uint32_t n_fixed,
                                 const uint32_t *n_dev, float *out, uint32_t *err, int device, cudaStream_t st) {
-  const size_t smem = ws_smem(P.hidden);
-  NR_CHECK_CUDA(cudaFuncSetAttribute(field_ws_kernel<T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  field_ws_kernel<T, MODE><<<num_sms(device), kWsThreads, smem, st>>>(P, blob, in, n_fixed, n_dev, out, err);
-  NR_CHECK_CUDA(cudaGetLastError());
-  return NR_OK;
+  if (MODE == kModeRender && P.whole_box)
+    return launch_ws_kernel<T, MODE, MODE == kModeRender>(P, blob, in, n_fixed, n_dev, out, err, device, st);
+  return launch_ws_kernel<T, MODE, false>(P, blob, in, n_fixed, n_dev, out, err, device, st);
 }
 
 nr_status launch_field_ws(const FieldParams &P, nr_dtype mlp_dtype, int mode, const float4 *in, uint32_t n_fixed,

@@ -166,6 +166,12 @@ __global__ void __launch_bounds__(kF32MaxThreads<MODE>, 1) field_f32_kernel(Fiel
       if (lane == 0) reinterpret_cast<uint32_t *>(out)[tile] = 0u;
       continue;
     }
+    if (MODE == kModeRender && !__any_sync(0xffffffffu, valid && S != 0.f)) {
+      // no bone reaches any of the tile's samples: S = 0, alpha = (..) min(S, 1) = 0, and they add
+      // nothing to their rays
+      if (valid) reinterpret_cast<float4 *>(out)[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+      continue;
+    }
     if (P.res_enabled) {
       pos_enc(P, s0, s1, s2, put_g);
       residual_f32(P, sW, sB1, g, h, o);

@@ -665,6 +665,7 @@ FieldParams field_params(const nr_subject *s, const nr_render_opts *o) {
   P.tlay = s->tlay;
   P.G = s->d_G;
   P.bias1 = s->d_bias1;
+  P.whole_box = (o && !o->use_occupancy) ? 1 : 0;
   P.bone_box = (o && !(o->flags & NR_RENDER_ALL_BONES)) ? s->bone_box : nullptr;
   P.fp8_blob = s->fp8_blob;
   P.fp8_scales = s->fp8_scales;
