@@ -27,26 +27,18 @@ __global__ void __launch_bounds__(256) march_kernel(CamParams cam, MarchParams m
   const bool hit = valid && ray_pixel(cam, r, u, v) && ray_setup(cam, o, mp.bmin, mp.bmax, u, v, d, lo, hi);
   const uint32_t S = cam.n_samples;
   const float D = __fdiv_rn(__fsub_rn(hi, lo), (float)S);
-  const int G = mp.grid;
-  float h[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) h[k] = __fdiv_rn(__fsub_rn(mp.bmax[k], mp.bmin[k]), (float)G);
+  const CellGrid grid(mp);
   auto live = [&](uint32_t i, float x[3]) -> bool {
     const float t = __fadd_rn(lo, __fmul_rn(__fadd_rn((float)i, 0.5f), D));
 #pragma unroll
     for (int k = 0; k < 3; ++k) x[k] = __fadd_rn(o[k], __fmul_rn(t, d[k]));
     if (!mp.bits) return true;
-    int c[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      int ck = (int)floorf(__fdiv_rn(__fsub_rn(x[k], mp.bmin[k]), h[k]));
-      c[k] = min(max(ck, 0), G - 1);
-    }
-    const uint32_t cell = ((uint32_t)c[2] * G + (uint32_t)c[1]) * G + (uint32_t)c[0];
+    const uint32_t cell = grid.cell(x);
     return (__ldg(mp.bits + (cell >> 5)) >> (cell & 31)) & 1u;
   };
   uint32_t count = 0;
   if (hit) {
+#pragma unroll 4
     for (uint32_t i = 0; i < S; ++i) {
       float x[3];
       count += live(i, x) ? 1u : 0u;
@@ -321,10 +313,7 @@ __global__ void __launch_bounds__(256) march_round_kernel(CamParams cam, MarchPa
                       ray_setup(cam, o, mp.bmin, mp.bmax, u, v, d, lo, hi);
   const uint32_t S = cam.n_samples;
   const float D = __fdiv_rn(__fsub_rn(hi, lo), (float)S);
-  const int G = mp.grid;
-  float h[3];
-#pragma unroll
-  for (int q = 0; q < 3; ++q) h[q] = __fdiv_rn(__fsub_rn(mp.bmax[q], mp.bmin[q]), (float)G);
+  const CellGrid grid(mp);
   auto pos = [&](uint32_t i, float x[3]) {
     const float t = __fadd_rn(lo, __fmul_rn(__fadd_rn((float)i, 0.5f), D));
 #pragma unroll
@@ -333,13 +322,7 @@ __global__ void __launch_bounds__(256) march_round_kernel(CamParams cam, MarchPa
   auto live = [&](uint32_t i, float x[3]) -> bool {
     pos(i, x);
     if (!mp.bits) return true;
-    int c[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      int cq = (int)floorf(__fdiv_rn(__fsub_rn(x[q], mp.bmin[q]), h[q]));
-      c[q] = min(max(cq, 0), G - 1);
-    }
-    const uint32_t cell = ((uint32_t)c[2] * G + (uint32_t)c[1]) * G + (uint32_t)c[0];
+    const uint32_t cell = grid.cell(x);
     return (__ldg(mp.bits + (cell >> 5)) >> (cell & 31)) & 1u;
   };
   const uint32_t i0 = st0 & ~kRayDone;
@@ -348,12 +331,20 @@ __global__ void __launch_bounds__(256) march_round_kernel(CamParams cam, MarchPa
   if (active) {
     float x[3];
     uint32_t i = i0;
-    for (; i < S && count < k; ++i) {
-      const bool lv = live(i, x);
-      count += lv ? 1u : 0u;
-      const uint32_t e = i - i0;
-      if (lv && e < 64u) m0 |= 1ull << e;
-      else if (lv && e < 128u) m1 |= 1ull << (e - 64u);
+    while (i < S && count < k) {   // four slots' bits loaded at a time, taken up to the k-th live one
+      uint32_t four = 0u;
+#pragma unroll
+      for (uint32_t q = 0; q < 4; ++q)
+        if (i + q < S) four |= (live(i + q, x) ? 1u : 0u) << q;
+#pragma unroll
+      for (uint32_t q = 0; q < 4; ++q)
+        if (i < S && count < k) {
+          const uint32_t lv = (four >> q) & 1u, e = i - i0;
+          count += lv;
+          if (e < 64u) m0 |= (uint64_t)lv << e;
+          else if (e < 128u) m1 |= (uint64_t)lv << (e - 64u);
+          ++i;
+        }
     }
     i_end = i;
   }

@@ -21,6 +21,13 @@ struct CamParams {
   uint32_t patch_cols;           // rays in patches of 8 x 4 pixels: patches per row; 0: in row order
 };
 
+struct MarchParams {
+  float bmin[3], bmax[3];
+  int grid;
+  const uint32_t *bits;          // posed occupancy bitfield, or NULL to keep every sample
+  uint32_t ray0, ray_end;        // rays of this chunk
+};
+
 // Rays are numbered in patches of 8 x 4 pixels where the image allows it, so that a warp's 32 rays
 // are neighbours both ways: at one depth their samples then lie in one or a few cells of the weight
 // volume and of the coarser hash levels.  r's pixel; false for a number past the image's edge.
@@ -36,6 +43,35 @@ __device__ __forceinline__ bool ray_pixel(const CamParams &c, uint32_t r, uint32
   return u < c.width && v < c.height;
 }
 
+// The occupancy cell of a point: floor((x - bmin) / h) per axis, h = (bmax - bmin) / G, clamped to
+// the grid, the quotient correctly rounded.  Where every h is a power of two (a 2 m box and a grid
+// of 32 to 256 cells) the division is a multiplication by its exact reciprocal, which rounds to
+// the same value: three divisions were half of a slot test's instructions.
+struct CellGrid {
+  float bmin[3], h[3], inv[3];
+  int G;
+  bool exact;
+  __device__ __forceinline__ CellGrid(const MarchParams &mp) : G(mp.grid), exact(true) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      bmin[k] = mp.bmin[k];
+      h[k] = __fdiv_rn(__fsub_rn(mp.bmax[k], mp.bmin[k]), (float)mp.grid);
+      inv[k] = __fdiv_rn(1.f, h[k]);
+      const uint32_t b = __float_as_uint(h[k]), e = b >> 23;
+      exact = exact && (b & 0x7fffffu) == 0u && e > 32u && e < 222u;   // far from subnormal and infinite
+    }
+  }
+  __device__ __forceinline__ uint32_t cell(const float x[3]) const {
+    int c[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float d = __fsub_rn(x[k], bmin[k]);
+      c[k] = min(max((int)floorf(exact ? __fmul_rn(d, inv[k]) : __fdiv_rn(d, h[k])), 0), G - 1);
+    }
+    return ((uint32_t)c[2] * G + (uint32_t)c[1]) * G + (uint32_t)c[0];
+  }
+};
+
 // The samples of a warp's 32 rays lie in the queue step by step: the first samples of all rays
 // that have one, then the second ones, and so on, from `base`; neighbouring lanes of the field
 // kernel thus hold neighbouring rays' samples at one depth instead of one ray's samples in depth.
@@ -49,13 +85,6 @@ struct StepQueue {
     at += __popc(m);
     return p;
   }
-};
-
-struct MarchParams {
-  float bmin[3], bmax[3];
-  int grid;
-  const uint32_t *bits;          // posed occupancy bitfield, or NULL to keep every sample
-  uint32_t ray0, ray_end;        // rays of this chunk
 };
 
 // Slab clip of the ray o + t d against [bmin, bmax] starting from
