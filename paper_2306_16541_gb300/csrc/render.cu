@@ -381,36 +381,37 @@ __global__ void __launch_bounds__(256) march_round_kernel(CamParams cam, MarchPa
 }
 
 // Folds a round's samples into each active ray's (C, T); retires rays below t_min or out of slots.
-__global__ void __launch_bounds__(256) composite_round_kernel(const uint2 *__restrict__ ray_range,
+// The last round also writes the pixels of all rays (out not NULL).
+__global__ void __launch_bounds__(256) composite_round_kernel(CamParams cam, uint32_t ray0,
+                                                              const uint2 *__restrict__ ray_range,
                                                               const float4 *__restrict__ so, uint32_t n_rays,
                                                               float t_min, uint32_t S, float4 *__restrict__ state,
-                                                              uint32_t *__restrict__ next, uint32_t *__restrict__ counter) {
+                                                              uint32_t *__restrict__ next, uint32_t *__restrict__ counter,
+                                                              float bg0, float bg1, float bg2,
+                                                              float4 *__restrict__ out) {
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r == 0) *counter = 0u;   // the round's field launch has read it: cleared for the next march
   const uint32_t nx = r < n_rays ? next[r] : kRayDone;
   const bool open = !(nx & kRayDone);
   RayFold F{0.f, 0.f, 0.f, 1.f, false};
-  uint2 rr = r < n_rays ? ray_range[r] : make_uint2(0u, 0u);   // a retired ray's count is 0
-  if (open) {
+  const uint2 rr = r < n_rays ? ray_range[r] : make_uint2(0u, 0u);   // a retired ray's count is 0
+  if (open || (out && r < n_rays)) {
     const float4 c = state[r];
     F = RayFold{c.x, c.y, c.z, c.w, false};
   }
   fold_steps(so, rr, t_min, F);
+  uint32_t u, v;
+  if (out) {
+    if (r < n_rays && ray_pixel(cam, ray0 + r, u, v))
+      out[(size_t)v * cam.width + u] = make_float4(fmaf(F.T, bg0, F.c0), fmaf(F.T, bg1, F.c1), fmaf(F.T, bg2, F.c2), 1.f - F.T);
+    return;
+  }
   if (!open) return;
   state[r] = make_float4(F.c0, F.c1, F.c2, F.T);
   if (F.done || nx >= S) next[r] = nx | kRayDone;
 }
 
 __global__ void add_u32_kernel(uint32_t *__restrict__ acc, const uint32_t *__restrict__ v) { *acc += *v; }
-
-__global__ void finalize_rays_kernel(CamParams cam, uint32_t ray0, const float4 *__restrict__ state, uint32_t n_rays,
-                                     float bg0, float bg1, float bg2, float4 *__restrict__ out) {
-  const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-  uint32_t u, v;
-  if (r >= n_rays || !ray_pixel(cam, ray0 + r, u, v)) return;
-  const float4 c = state[r];
-  out[(size_t)v * cam.width + u] = make_float4(fmaf(c.w, bg0, c.x), fmaf(c.w, bg1, c.y), fmaf(c.w, bg2, c.z), 1.f - c.w);
-}
 
 int num_sms(int device) {
   static int cached[64] = {0};
@@ -617,19 +618,15 @@ nr_status render_rays(const nr_subject *s, const FieldParams &P, const uint32_t 
         return r;
       NR_CHECK_CUDA(mark(1));
       if (rounds)
-        composite_round_kernel<<<nb, 256, 0, st>>>(w.ray_range, w.samp_out, nr_, opts->t_min, S, w.state, w.next,
-                                                   w.counter);
+        composite_round_kernel<<<nb, 256, 0, st>>>(C, r0, w.ray_range, w.samp_out, nr_, opts->t_min, S, w.state,
+                                                   w.next, w.counter, cam->bg[0], cam->bg[1], cam->bg[2],
+                                                   round + 1 == n_rounds ? dst : nullptr);
       else
         composite_kernel<<<nb, 256, 0, st>>>(C, r0, w.ray_range, w.samp_out, nr_, opts->t_min, cam->bg[0], cam->bg[1],
                                              cam->bg[2], dst);
       NR_CHECK_CUDA(cudaGetLastError());
       NR_CHECK_CUDA(mark(2));
       count_launches(3);
-    }
-    if (rounds) {
-      finalize_rays_kernel<<<nb, 256, 0, st>>>(C, r0, w.state, nr_, cam->bg[0], cam->bg[1], cam->bg[2], dst);
-      NR_CHECK_CUDA(cudaGetLastError());
-      count_launches(1);
     }
   }
   return NR_OK;
