@@ -86,7 +86,7 @@ struct TrainDev {
   int n_frames;
   Rows rw;
   float *dG;              // [F][24][12] dL/dG of every frame (pose refiner), or NULL
-  int dG_smem;            // 1: the block sums dG in shared memory first
+  int dG_acc;             // 1: the blocks sum dG in their accumulators first, behind the frame biases
   FragLay fl;             // shared-memory layout of the weights
   float *pred;            // [n][3] composited colours out, or NULL
   const float *grad_rgb;  // [n][3] dL/dC from the caller, or NULL (MSE against target)
@@ -620,10 +620,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams
   extern __shared__ float4 smem4[];
   float *sW = reinterpret_cast<float *>(smem4);
   float *tiles = sW + T.fl.total;                      // a tile per warp
-  float *sdG = tiles + (blockDim.x >> 5) * kTileFloats;   // [F][24][12] when T.dG_smem
   stage_frag_weights(P.blob, P.lay, T.fl, P.hidden, sW);
-  if (T.dG && T.dG_smem)
-    for (int i = threadIdx.x; i < T.n_frames * kBones * 12; i += blockDim.x) sdG[i] = 0.f;
   __syncthreads();
   const BlobLayout &Ly = P.lay;                        // the gradient accumulators' layout
   const FragLay &W = T.fl;
@@ -634,6 +631,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams
   float *img = T.scratch + ((size_t)blockIdx.x * (blockDim.x >> 5) + warp) * R.total * kTileRow;
   float *acc = T.wacc + (size_t)blockIdx.x * T.acc_floats;
   float *accF = acc + Ly.total;                        // per-frame first-layer bias gradients [F][64]
+  float *accG = T.dG_acc ? accF + T.n_frames * kWidth : T.dG;   // dL/dG [F][24][12]
   const int H = P.hidden;
   const uint32_t n = T.n_rays * T.S;
   const uint32_t step = gridDim.x * blockDim.x;
@@ -946,7 +944,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams
         // tensor-core product (M = 72 rows of dp in 16-row tiles, N = 4 columns padded to 8,
         // K = the 32 samples; m16n8k8 TF32, three products per step)
         const int g = lane >> 2, t = lane & 3;
-        float *dst = (T.dG_smem ? sdG : T.dG) + (size_t)f0 * kBones * 12;
+        float *dst = accG + (size_t)f0 * kBones * 12;
         uint32_t bh[4][2], bl[4][2];   // B[s][c] = (x, y, z, 1)[c] of sample s, zero for c >= 4
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
@@ -990,22 +988,17 @@ __global__ void __launch_bounds__(kTrainThreads, 1) train_bwd_kernel(FieldParams
           const int fr = __shfl_sync(0xffffffffu, fl, sI);
           if (fr < 0) break;
           if (fr != cur) {
-            if (cur >= 0 && v != 0.f) atomicAdd((T.dG_smem ? sdG : T.dG) + cur * kBones * 12 + o, v);
+            if (cur >= 0 && v != 0.f) atomicAdd(accG + cur * kBones * 12 + o, v);
             cur = fr;
             v = 0.f;
           }
           v = fmaf(dpr[sI], c < 3 ? xr[sI] : 1.f, v);
         }
-        if (cur >= 0 && v != 0.f) atomicAdd((T.dG_smem ? sdG : T.dG) + cur * kBones * 12 + o, v);
+        if (cur >= 0 && v != 0.f) atomicAdd(accG + cur * kBones * 12 + o, v);
       }
       }
     }
     __syncwarp();
-  }
-  if (T.dG && T.dG_smem) {
-    __syncthreads();
-    for (int i = threadIdx.x; i < T.n_frames * kBones * 12; i += blockDim.x)
-      if (sdG[i] != 0.f) atomicAdd(T.dG + i, sdG[i]);
   }
 }
 
@@ -1166,7 +1159,11 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
   P.bone_box = nullptr;   // training differentiates every bone channel
   const size_t n = (size_t)b->n_rays * b->n_samples;
   const int blocks = num_sms(s->device);
-  const int A = s->lay.total + (int)s->n_frames * kWidth;
+  // dL/dG of a few frames is summed per block first, in the block's accumulator: in shared memory it
+  // took the place of four warps' tiles
+  const bool dG_acc = refine && s->n_frames <= 16;
+  const size_t n_dG = (size_t)s->n_frames * kBones * 12;
+  const int A = s->lay.total + (int)s->n_frames * kWidth + (dG_acc ? (int)n_dG : 0);
   if (n > s->tw_samples) {              // the three per-sample buffers grow together
     size_t c0 = 0, c1 = 0, c2 = 0;
     if (s->t_samp) cudaFree(s->t_samp);
@@ -1185,13 +1182,10 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
   if ((r = grow(s->t_live, s->tw_live, ((size_t)b->n_rays * b->n_samples + 31) / 32)) != NR_OK) return r;
   const Rows rows = make_rows((int)s->hidden);
   const FragLay fl = frag_layout((int)s->hidden);
-  const size_t n_dG = (size_t)s->n_frames * kBones * 12;
-  const bool dG_smem = refine && s->n_frames <= 16;
   // the warps whose tiles fit beside the weights (sixteen with two hidden layers, eleven with four)
-  const size_t smem_w = sizeof(float) * fl.total, smem_g = dG_smem ? sizeof(float) * n_dG : 0;
+  const size_t smem_w = sizeof(float) * fl.total;
   const size_t tile_b = kTileFloats * sizeof(float);
-  const int warps_f = (int)std::min<size_t>(kTrainThreads / 32, (kTrainSmem - smem_w) / tile_b);
-  const int warps_max = (int)std::min<size_t>(kTrainThreads / 32, (kTrainSmem - smem_w - smem_g) / tile_b);
+  const int warps_max = (int)std::min<size_t>(kTrainThreads / 32, (kTrainSmem - smem_w) / tile_b);
   // a step whose rays fit a block whole runs forward, compositing and backward in one kernel
   // (train_bwd_kernel<true>) over groups of 32 warps / S rays; else the forward and the
   // compositing adjoint run first
@@ -1263,7 +1257,7 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
   T.n_frames = (int)s->n_frames;
   T.rw = rows;
   T.dG = refine ? s->f_dG : nullptr;
-  T.dG_smem = dG_smem ? 1 : 0;
+  T.dG_acc = dG_acc ? 1 : 0;
   T.fl = fl;
   T.pred = b->pred_rgb;
   T.grad_rgb = fwd_only ? nullptr : b->grad_rgb;
@@ -1273,9 +1267,9 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
                                                                      s->bmax[1], s->bmax[2]);
   NR_CHECK_CUDA(cudaGetLastError());
   if (!fused) {
-    const size_t smem_f = smem_w + warps_f * tile_b;
+    const size_t smem_f = smem_w + warps_max * tile_b;
     NR_CHECK_CUDA(cudaFuncSetAttribute(train_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_f));
-    train_fwd_kernel<<<blocks, 32 * warps_f, smem_f, st>>>(P, T);
+    train_fwd_kernel<<<blocks, 32 * warps_max, smem_f, st>>>(P, T);
     NR_CHECK_CUDA(cudaGetLastError());
     train_composite_kernel<<<(b->n_rays + 255) / 256, 256, 0, st>>>(T);
     NR_CHECK_CUDA(cudaGetLastError());
@@ -1289,7 +1283,7 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
     }
     return NR_OK;
   }
-  const size_t smem_b = smem_w + smem_g + warps_b * tile_b;
+  const size_t smem_b = smem_w + warps_b * tile_b;
   if (fused) {
     NR_CHECK_CUDA(
         cudaFuncSetAttribute(train_bwd_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b));
@@ -1323,7 +1317,8 @@ extern "C" nr_status nr_train_step(nr_subject *s, const nr_train_batch *b, float
   scatter_mlp_kernel<<<(sa.m.n_mlp + 255) / 256, 256, 0, st>>>(s->t_red, sa, s->g_mlp);
   NR_CHECK_CUDA(cudaGetLastError());
   launched += 5;   // samples, backward, reduction, two scatters
-  if (refine && (r = launch_refine_bwd(s, s->f_omega, 3 * kBones, s->f_root, 3, (int)s->n_frames, s->f_dG,
+  if (refine && (r = launch_refine_bwd(s, s->f_omega, 3 * kBones, s->f_root, 3, (int)s->n_frames,
+                                       dG_acc ? s->t_red + s->lay.total + s->n_frames * kWidth : s->f_dG,
                                        s->t_red + s->lay.total, s->g_ref, st)) != NR_OK)
     return r;
   if (s->cnn_on && (r = cnn_backward(s, st)) != NR_OK) return r;   // dL/dW^c -> CNN_skel
