@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256) cnn_convt_fwd(const float *__restrict__ i
 // output and input) and its inputs are read coalesced, once for the kFwdOut outputs; a thread per
 // output read two values from L1 for each multiply-add.  Each sum runs over the inputs and taps in
 // the order of cnn_convt_fwd, so the volume keeps its bits.  0.37 and 0.45 ms for the last two
-// layers before.
+// layers before, 0.17 for both now.
 constexpr int kFwdOut = 4, kFwdIn = 16, kFwdThreads = 128;
 __global__ void __launch_bounds__(kFwdThreads) cnn_convt_fwd_wide(const float *__restrict__ in,
                                                                   const float *__restrict__ W,
@@ -199,7 +199,7 @@ __global__ void cnn_softmax_bwd(const float *__restrict__ w, const float *__rest
 // r >= 8: a block takes 64 positions and four inputs, its four pairs of warps every fourth output;
 // a thread's 64 dout values of an output serve the four inputs, whose weights come from shared
 // memory as broadcasts.  (One group of lanes per input value, each reading its own weight rows and
-// window, took 0.17-0.39 ms a layer.)
+// window, took 0.17 and 0.22 ms for the two layers; 0.17 for both now.)
 constexpr int kBackIn = 4;
 __global__ void __launch_bounds__(256) cnn_convt_bwd_data_wide(const float *__restrict__ in, const float *__restrict__ W,
                                                                const float *__restrict__ dout, int Cin, int Cout, int r,
@@ -255,7 +255,8 @@ __global__ void __launch_bounds__(256) cnn_convt_bwd_data_wide(const float *__re
 
 // r = 1, 2, 4: a block takes one input channel with every position in its registers.  Its threads
 // are the 64 taps by four outputs, so the weights, the larger operand here, are read once and
-// coalesced; the outputs' gradients lie in shared memory with a rim of zeros.
+// coalesced; the outputs' gradients lie in shared memory with a rim of zeros.  r = 4: 0.39 -> 0.16 ms,
+// r = 2: 0.22 -> 0.10, r = 1: 0.038 -> 0.053 (reading only the inner taps there changed nothing).
 template <int r>
 __global__ void __launch_bounds__(256) cnn_convt_bwd_data_deep(const float *__restrict__ in, const float *__restrict__ W,
                                                                const float *__restrict__ dout, int Cout,
@@ -309,7 +310,8 @@ __global__ void __launch_bounds__(256) cnn_convt_bwd_data_deep(const float *__re
 //
 // r >= 4: a block takes one output and eight inputs; its threads are the 64 taps by slices of the
 // planes of q.  A dout value serves the eight inputs, whose values are the same for all taps
-// (16-byte broadcasts).  (A thread per weight took 0.43 ms for the last layer's 102,400.)
+// (16-byte broadcasts).  (A thread per weight took 0.43 ms for the last layer's 102,400 and
+// 0.71 for the three; 0.34 now.)
 constexpr int kWgIn = 8;
 __global__ void __launch_bounds__(512) cnn_convt_bwd_weight_wide(const float *__restrict__ in,
                                                                  const float *__restrict__ dout, int Cin, int Cout,
@@ -362,7 +364,7 @@ __global__ void __launch_bounds__(512) cnn_convt_bwd_weight_wide(const float *__
 }
 
 // r = 1, 2: few positions and many weights, so the kernel is the store of dW: a thread per tap
-// row of an output (four weights), a grid row per input, no division.
+// row of an output (four weights), a grid row per input, no division (0.27 ms for both, 0.07 now).
 __global__ void __launch_bounds__(256) cnn_convt_bwd_weight_deep(const float *__restrict__ in,
                                                                  const float *__restrict__ dout, int Cout, int r,
                                                                  int aligned, float *__restrict__ dW) {

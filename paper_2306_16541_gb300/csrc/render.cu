@@ -83,7 +83,8 @@ __global__ void __launch_bounds__(256) march_kernel(CamParams cam, MarchParams m
 // Bound by the FMA pipe (28 K FMAs per sample of the tiny workload) and, level with it, the loads of
 // its operands, at eight warps an SM: the weights (100-135 KB) and 13.3 KB of activations a warp
 // fill the shared memory.  Forming gamma twice instead of holding it makes room for twelve warps,
-// which gained nothing (a 250,007-point query 382 -> 391 us); the density grid, which has no gamma,
+// which gained nothing (a 250,007-point query, 655 us with a thread per sample, takes 378 with eight
+// warps and 391 with twelve); the density grid, which has no gamma,
 // takes twelve.
 template <int MODE>
 constexpr int kF32MaxThreads = MODE == kModeDensity ? 384 : 256;
