@@ -173,7 +173,7 @@ struct nr_subject {
   bool fp8_ready = false;
   uint8_t *t5_bf16 = nullptr, *t5_f16 = nullptr, *t5_fp8 = nullptr;
   uint32_t *t5_err = nullptr;
-  uint32_t *h_err = nullptr;         // pinned copy of *t5_err
+  uint32_t *h_err = nullptr;         // pinned copy of *t5_err, allocated with the subject
   bool t5_ready = false;
   // current pose
   bool pose_set = false;

@@ -468,8 +468,8 @@ bool path_uses_tcgen05(const nr_render_opts *o, int path) {
 
 nr_status check_field_timeouts(nr_subject *s, cudaStream_t st) {
   if (!s->t5_err) return NR_OK;
-  // into pinned memory: a copy to the stack goes through the driver's staging buffer
-  if (!s->h_err) NR_CHECK_CUDA(cudaMallocHost((void **)&s->h_err, sizeof(uint32_t)));
+  // into pinned memory, allocated with the subject (nr_render_static must not allocate): a copy to
+  // the stack goes through the driver's staging buffer
   NR_CHECK_CUDA(cudaMemcpyAsync(s->h_err, s->t5_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
   NR_CHECK_CUDA(cudaStreamSynchronize(st));
   const uint32_t word = *s->h_err;

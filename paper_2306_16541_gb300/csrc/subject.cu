@@ -839,6 +839,7 @@ extern "C" nr_status nr_create_subject(const nr_subject_desc *d, void *stream, n
   }
 #undef ALLOC
   cudaError_t e;
+  if ((e = cudaMallocHost((void **)&s->h_err, sizeof(uint32_t))) != cudaSuccess) return fail(e, "cudaMallocHost h_err");
 #define H2D(dst, src, bytes)                                                   \
   e = cudaMemcpyAsync((dst), (src), (bytes), cudaMemcpyHostToDevice, st);      \
   if (e != cudaSuccess) return fail(e, "cudaMemcpyAsync " #dst);
