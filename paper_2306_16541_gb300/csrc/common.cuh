@@ -104,7 +104,8 @@ struct FieldParams {
   const uint8_t *t5_bf16, *t5_f16;   // swizzled K-major weight blobs of the tcgen05 path (field_t5.cu)
   const uint8_t *t5_fp8;             // the same layout in e4m3 with the fp8 tier's scales (field_fp8.cu)
   uint32_t *t5_err;                  // set by the tcgen05 path when a bounded wait gives up
-  int whole_box;                     // a render without occupancy: samples all over the box
+  int whole_box;                     // a render without occupancy (samples all over the box): the
+                                     // samples of a ray in one launch; else 0
   const float *bone_box;             // [24][6] per-bone support box in volume-index units, or NULL
   // occupancy from the field's density (kModeDensity / kModePose of the FP32 kernel)
   int occ_grid;                      // cells per axis

@@ -557,7 +557,7 @@ uint32_t round_samples(const nr_camera *cam, const nr_render_opts *opts) {
   return std::min<uint32_t>(cam->n_samples, std::max<uint32_t>(16u, (cam->n_samples + 3) / 4));
 }
 
-nr_status render_rays(const nr_subject *s, const FieldParams &P, const uint32_t *bits, const nr_camera *cam,
+nr_status render_rays(const nr_subject *s, const FieldParams &params, const uint32_t *bits, const nr_camera *cam,
                       const nr_render_opts *opts, const FrameWork &w, float4 *dst, cudaStream_t st, int mma_path,
                       Prof *prof) {
   const CamParams C = cam_params(cam, UINT64_MAX);   // any number of rays: they are taken in chunks
@@ -565,6 +565,8 @@ nr_status render_rays(const nr_subject *s, const FieldParams &P, const uint32_t 
   const uint32_t S = cam->n_samples;
   const uint32_t k = round_samples(cam, opts);
   const bool rounds = k < S || opts->t_min > 0.f;
+  FieldParams P = params;
+  if (P.whole_box) P.whole_box = (int)k;
   uint32_t chunk = (uint32_t)std::min<uint64_t>(std::min<uint64_t>(n_rays, w.cap_rays),
                                                 std::max<uint64_t>(1, w.cap_samples / k));
   if (chunk > 32 && chunk < n_rays) chunk &= ~31u;     // whole patches

@@ -119,7 +119,8 @@ extern "C" nr_status nr_render_static(nr_subject *s, const nr_camera *cam, const
   const int path = render_path(opts);
   const bool t5 = path_uses_tcgen05(opts, path);
   if (t5 && (r = prepare_t5(s, st)) != NR_OK) return r;
-  const FieldParams P = field_params(s, opts);
+  FieldParams P = field_params(s, opts);
+  if (P.whole_box) P.whole_box = (int)cam->n_samples;
   const CamParams C = cam_params(cam, n_rays);   // patches only where they cover the image exactly
   MarchParams mp{};
   for (int k = 0; k < 3; ++k) {
