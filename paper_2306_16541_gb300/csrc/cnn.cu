@@ -99,7 +99,9 @@ __global__ void __launch_bounds__(256) cnn_convt_fwd(const float *__restrict__ i
 // output and input) and its inputs are read coalesced, once for the kFwdOut outputs; a thread per
 // output read two values from L1 for each multiply-add.  Each sum runs over the inputs and taps in
 // the order of cnn_convt_fwd, so the volume keeps its bits.  0.37 and 0.45 ms for the last two
-// layers before, 0.17 for both now.
+// layers before, 0.17 for both now.  A tap outside the input is a product with zero (as in the
+// gradients below): weights are finite when they are installed, and one that has become infinite
+// since makes the rim NaN along with the voxels that it reaches.
 constexpr int kFwdOut = 4, kFwdIn = 16, kFwdThreads = 128;
 __global__ void __launch_bounds__(kFwdThreads) cnn_convt_fwd_wide(const float *__restrict__ in,
                                                                   const float *__restrict__ W,
@@ -253,10 +255,28 @@ __global__ void __launch_bounds__(256) cnn_convt_bwd_data_wide(const float *__re
   }
 }
 
-// r = 1, 2, 4: a block takes one input channel with every position in its registers.  Its threads
+// r = 1: an input sees the eight outputs through the inner taps (1 and 2 of each axis); the outer
+// taps reach nothing and their weights are not read.  `split` lanes per input (outputs o = j,
+// j + split, ...), summed over shuffles.  0.025 ms for 1024 x 512 channels (0.053 as below).
+__global__ void __launch_bounds__(256) cnn_convt_bwd_data_first(const float *__restrict__ in, const float *__restrict__ W,
+                                                                const float *__restrict__ dout, int Cin, int Cout,
+                                                                int split, float *__restrict__ din) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, i = t / split, j = t % split;
+  float acc = 0.f;
+  if (i < Cin)
+    for (int o = j; o < Cout; o += split) {
+      const float *wi = W + ((size_t)i * Cout + o) * 64, *go = dout + (size_t)o * 8;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) acc = fmaf(wi[((u >> 2) + 1) * 16 + (((u >> 1) & 1) + 1) * 4 + (u & 1) + 1], go[u], acc);
+    }
+  for (int off = split >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+  if (i < Cin && j == 0) din[i] = acc * leaky_grad(in[i]);
+}
+
+// r = 2, 4: a block takes one input channel with every position in its registers.  Its threads
 // are the 64 taps by four outputs, so the weights, the larger operand here, are read once and
 // coalesced; the outputs' gradients lie in shared memory with a rim of zeros.  r = 4: 0.39 -> 0.16 ms,
-// r = 2: 0.22 -> 0.10, r = 1: 0.038 -> 0.053 (reading only the inner taps there changed nothing).
+// r = 2: 0.22 -> 0.10.
 template <int r>
 __global__ void __launch_bounds__(256) cnn_convt_bwd_data_deep(const float *__restrict__ in, const float *__restrict__ W,
                                                                const float *__restrict__ dout, int Cout,
@@ -533,8 +553,10 @@ nr_status cnn_backward(nr_subject *s, cudaStream_t st) {
       cnn_convt_bwd_data_deep<4><<<cin, 256, 0, st>>>(x, w, d0, cout, d1);
     else if (r == 2)
       cnn_convt_bwd_data_deep<2><<<cin, 256, 0, st>>>(x, w, d0, cout, d1);
-    else
-      cnn_convt_bwd_data_deep<1><<<cin, 256, 0, st>>>(x, w, d0, cout, d1);
+    else {
+      const int sp = cnn_split(cin, cout);
+      cnn_convt_bwd_data_first<<<blocks_for((size_t)cin * sp), 256, 0, st>>>(x, w, d0, cin, cout, sp, d1);
+    }
     std::swap(d0, d1);
     launched += 3;
   }

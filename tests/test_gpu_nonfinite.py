@@ -89,3 +89,34 @@ def test_a_bad_output_weight_shows(bits, tc):
             assert not np.isfinite(loss) and not torch.isfinite(pred).any()
     finally:
         sub.close()
+
+
+def test_a_bad_weight_of_a_tap_that_reaches_nothing_stays_alone():
+    """The generator's first transposed convolution takes one voxel to 2^3: the outer taps of its 4^3
+    kernels reach nothing, so their values enter neither the volume nor any gradient."""
+    nr = nrmod()
+    s = synth.subject(421)
+    layers = synth.cnn_layers(422, SMALL, last_std=0.3)
+    frames = synth.training_frames(423, 1, res=32)
+    sub = nr.Subject(s)
+    try:
+        sub.set_weight_cnn(layers, synth.cnn_latent(424), _prior(s))
+        sub.set_frames(frames["axis_angle"], frames["root_t"], frames["cameras"])
+        n = 16
+        rays = [u32(a) for a in (np.zeros(n), np.full(n, 15), np.arange(8, 8 + n))]
+        p, g = sub.param(nr.NR_PARAM_CNN)
+        o = layers[0][0].size + layers[0][1].size
+        W1 = p[o:o + layers[1][0].size].view(*layers[1][0].shape)
+        grads = []
+        for bad in (False, True):
+            if bad:
+                W1[2, 3, 0, 1, 2] = float("inf")
+                W1[5, 7, 2, 3, 1] = float("nan")
+                sub.params_changed()
+            sub.train_step(*rays, None, 32, 3, grad_rgb=torch.full((n, 3), 0.1, device="cuda"), grad_only=True)
+            assert torch.isfinite(sub.param(nr.NR_PARAM_WVOL)[0]).all()
+            grads.append(g.cpu().numpy())
+    finally:
+        sub.close()
+    assert np.isfinite(grads[1]).all() and np.any(grads[0] != 0)
+    assert np.linalg.norm(grads[1] - grads[0]) <= 1e-4 * np.linalg.norm(grads[0])   # (sums by atomics)
