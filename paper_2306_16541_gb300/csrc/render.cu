@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(256) march_kernel(CamParams cam, MarchParams m
     const uint32_t w = Q.place(i < count);
     if (i < count) {
       float x[3];
-      while (!live(e, x)) ++e;
+      while (!live(e, x) && e < S) ++e;   // ends whatever has become of the bits since they were counted
       ++e;
       samp[w] = make_float4(x[0], x[1], x[2], D);
     }
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(256) march_round_kernel(CamParams cam, MarchPa
         pos(i0 + (low ? 0u : 64u) + (uint32_t)(__ffsll((long long)m) - 1), x);
         m &= m - 1u;
       } else {
-        while (!live(e, x)) ++e;
+        while (!live(e, x) && e < S) ++e;   // as in march_kernel
         ++e;
       }
       samp[w] = make_float4(x[0], x[1], x[2], D);
