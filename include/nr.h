@@ -203,6 +203,8 @@ typedef struct {
  * (rgb = sum_i T_i alpha_i c_i + T_final bg, a = 1 - T_final), where
  * alpha_i = (1 - exp(-sigma_i delta_i)) * min(S_i, 1) and S_i is the sum of
  * the bone weights at the sample (the likelihood augmentation of Sec. 4.4).
+ * A sample that no bone reaches (S_i = 0) adds nothing and may be left out, so
+ * a NaN of the field shows only on rays that meet a bone.
  * out_rgba may be a device or a host pointer; a host buffer is filled before
  * the call returns, a device buffer in stream order.  Errors: NR_ESTATE
  * before nr_set_pose; NR_EINVAL for bad sizes or options; NR_ENOMEM if the
@@ -456,8 +458,8 @@ nr_status nr_canonical_occupancy(nr_subject *s, uint32_t *bits_out);
                                  both MLPs as warp-level tensor-core layers at float32 accuracy
                                  (each product as three TF32 products of hi/lo parts) instead of
                                  CUDA-core FMAs.  The first such call allocates a scratch buffer of
-                                 one 212-float column per thread of one 512-thread block per SM
-                                 (66 MB on 152 SMs); nr_render_static refuses the flag
+                                 40 floats per thread of one 512-thread block per SM
+                                 (12 MB on 152 SMs); nr_render_static refuses the flag
                                  (NR_EUNSUPPORTED).  Ignored for the other dtypes and by the
                                  server, whose slots render concurrently. */
 

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kTf32Threads, 1) field_tf32_kernel(FieldParams
     float f0 = s0, f1 = s1, f2 = s2;
     if (MODE == kModeRender && !__any_sync(0xffffffffu, valid && S != 0.f)) {
       // no bone reaches any of the tile's samples: S = 0, alpha = (..) min(S, 1) = 0, and they add
-      // nothing to their rays
+      // nothing to their rays (of a finite field: a NaN shows only on rays that meet a bone)
       if (valid) reinterpret_cast<float4 *>(out)[j] = make_float4(0.f, 0.f, 0.f, 0.f);
       continue;
     }
@@ -121,7 +121,7 @@ nr_status launch_field_tf32(const FieldParams &P, int mode, const float4 *in, ui
     return NR_ESTATE;
   }
   const FragLay W = frag_layout(P.hidden);
-  // the warps whose tiles fit beside the weights (sixteen with two hidden layers, twelve with four)
+  // the warps whose tiles fit beside the weights (sixteen with two hidden layers, eleven with four)
   const size_t base = sizeof(float) * (W.total + kPoseSmem), tile_b = kTileFloats * sizeof(float);
   const int warps = (int)std::min<size_t>(kTf32Threads / 32, (227 * 1024 - base) / tile_b);
   const size_t smem = base + warps * tile_b;

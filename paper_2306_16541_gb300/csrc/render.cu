@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(kF32MaxThreads<MODE>, 1) field_f32_kernel(Fiel
     }
     if (MODE == kModeRender && !__any_sync(0xffffffffu, valid && S != 0.f)) {
       // no bone reaches any of the tile's samples: S = 0, alpha = (..) min(S, 1) = 0, and they add
-      // nothing to their rays
+      // nothing to their rays (of a finite field: a NaN shows only on rays that meet a bone)
       if (valid) reinterpret_cast<float4 *>(out)[j] = make_float4(0.f, 0.f, 0.f, 0.f);
       continue;
     }
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kF32MaxThreads<MODE>, 1) field_f32_kernel(Fiel
 }
 
 // Threads of an FP32 launch: the warps whose activations fit beside the weights (eight with two
-// hidden layers, six with four), and the launch itself.
+// hidden layers, seven with four), and the launch itself.
 static size_t f32_base_smem(const FieldParams &P) { return sizeof(float) * (P.lay.total + kPoseSmem + kWidth); }
 
 template <int MODE>

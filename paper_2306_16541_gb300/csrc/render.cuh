@@ -47,7 +47,9 @@ __device__ __forceinline__ bool ray_pixel(const CamParams &c, uint32_t r, uint32
 // The occupancy cell of a point: floor((x - bmin) / h) per axis, h = (bmax - bmin) / G, clamped to
 // the grid, the quotient correctly rounded.  Where every h is a power of two (a 2 m box and a grid
 // of 32 to 256 cells) the division is a multiplication by its exact reciprocal, which rounds to
-// the same value: three divisions were half of a slot test's instructions.
+// the same value: three divisions were half of a slot test's instructions.  Any other box divides (the
+// march of a 512 x 512 x 128 frame takes 0.14 ms with and 0.19 without; with early termination 0.17
+// and 0.21).
 struct CellGrid {
   float bmin[3], h[3], inv[3];
   int G;
@@ -176,7 +178,11 @@ nr_status render_frame(const nr_subject *s, const FieldParams &P, const uint32_t
 
 // max_slots: the ray numbers that the caller's buffers hold (at least width x height); patch order
 // is taken where its numbers, which cover the image in whole patches, stay within them and within
-// 1/8 over the pixels.
+// 1/8 over the pixels.  Only images of a few pixels one way lie beyond that line, and there the two
+// orders trade: over the whole box patches take 166 us and rows 180 at 1000 x 10 (1.2 numbers a
+// pixel), 290 and 268 at 20 x 1000 (1.2), 259 and 241 at 17 x 1000 (1.4), 131 and 133 at 1000 x 5
+// (1.6).  At 512 x 512 x 128 patches take 1.70 ms and rows 1.78 with an occupancy grid, 4.00 and 4.27
+// over the whole box.
 CamParams cam_params(const nr_camera *c, uint64_t max_slots);
 uint32_t ray_slots(const CamParams &c);                       // ray numbers of an image
 int render_path(const nr_render_opts *o);                     // the launch_field path the options select
